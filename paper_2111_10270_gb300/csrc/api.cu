@@ -342,6 +342,7 @@ int allocate_and_upload(fdog_instance* inst) {
         b.tile_first[c] = a.prefix + q + 2;
         b.tiles_total[c] = pre[q + 1];
         b.kmax[c] = d.kmax[c];
+        b.nodes_max[c] = d.nodes_max[c];
         q += 3;
     }
     auto two = [&](int32_t** dst, int32_t v) {

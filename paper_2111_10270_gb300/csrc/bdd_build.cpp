@@ -273,6 +273,8 @@ void build_templates(Decomposition& out) {
     for (size_t s = 0; s < out.shapes.size(); ++s) {
         const HostShape& h = out.shapes[s];
         int W = class_width(out.shape_cls[s]);
+        int& most = out.nodes_max[out.shape_cls[s]];
+        most = std::max(most, h.lstart.back());
         while (out.tpl.size() % 8) out.tpl.push_back(0);  // 16-byte aligned vector loads
         const int jit = out.shape_cls[s] == kJitClass ? jit_register_shape(h) : -1;
         ShapeDev d{h.k, static_cast<int32_t>(out.tpl.size()), W, jit};

@@ -96,6 +96,7 @@ int view_build(Engine& e, BatchView& v, const std::vector<fdog_instance*>& membe
             pre[i + 1] = pre[i] + cnt;
             first[i] = d.cls_tile_begin[c];
             b.kmax[c] = std::max(b.kmax[c], d.kmax[c]);
+            b.nodes_max[c] = std::max(b.nodes_max[c], d.nodes_max[c]);
             b.has_local[c] = b.has_local[c] || d.cls_has_local[c];
         }
         b.tile_prefix[c] = dints + q;

@@ -165,7 +165,8 @@ struct SweepArgs {
     const int32_t* first;   // [n_inst] first tile of this class in the instance
     int32_t n_inst;
     int32_t total;
-    int32_t kstride;        // shared-memory kernels: per-layer stride (>= longest row)
+    int32_t kstride;        // wide BDDs: longest row; long rows: most checkpoints of a row
+    int32_t nodes;          // wide BDDs: most nodes of a shape
     int32_t flags;          // evaluate at lambda + T (1) | write m0 and m1 (2)
     int32_t epi;            // update passes: layer stride of the per-warp staging for tile-local
                             // deferred sums (0: no tile of this launch has local variables)
@@ -226,6 +227,7 @@ struct Decomposition {
     int64_t n_bdds = 0, n_slots = 0, n_nodes = 0, slots_pad = 0;
     int64_t n_work = 0, n_wpos = 0, n_local_ent = 0;  // sizes of work, wpos, local_ent
     int kmax[kNumClasses] = {0};
+    int nodes_max[kNumClasses] = {0};  // most nodes of a shape of the class
     // Plan built on the device: var, csr_off, csr_pos, work, wpos, local_ent
     // and bdd_row exist only in device memory (d_* until the instance's arena
     // takes the first six; bdd_row stays in d_bdd_row) until a host consumer

@@ -368,7 +368,8 @@ inline int blocks_for(int total, int per_block, int cap) {
 }  // namespace
 
 int smem_max_layers(int width) {
-    // per warp: kTile columns x (lambda, T, W labels) floats per layer (staged kernels) or
+    // per warp: kTile columns x (lambda, T, at most W labels) floats per layer (wide BDDs; the running labels
+    // and terminals are above the 200 KB that this leaves for them) or
     // W labels per segment of kRegK layers (segmented kernels); at least one warp per block
     if (width <= kRegW) return kRegK * ((200 * 1024 - kEpiMaxK * 2 * kTile * 4) / (kTile * 4 * width));
     return (200 * 1024 - kEpiMaxK * 2 * kTile * 4) / (kTile * 4 * (2 + width));
@@ -384,15 +385,17 @@ cudaError_t launch_class(const DevBatch& b, int cls, int mode, int mm_flags, con
     const int W = class_width(cls);
     int wpb = cfg.warps_per_block;
     const bool seg = class_is_seg(cls);
-    // staged kernels: one row of state per layer; segmented kernels: one checkpoint per kRegK layers
+    // wide BDDs: two rows per layer, one per node, the running labels and the terminals;
+    // long rows: one checkpoint per kRegK layers
+    const int nodes = reg || seg ? 0 : b.nodes_max[cls];
     const int kstride = reg ? 0 : (seg ? (b.kmax[cls] + kRegK - 1) / kRegK : b.kmax[cls]);
     const int epi = ((mode == kFwdUpdate || mode == kBwdUpdate) && b.has_local[cls])
                         ? (b.kmax[cls] < kEpiMaxK ? b.kmax[cls] : kEpiMaxK) : 0;
-    const size_t per_warp =
-        (static_cast<size_t>(kstride) * (seg ? W : 2 + W) + static_cast<size_t>(epi) * 2) * kTile * sizeof(float);
+    const size_t rows = reg ? 0 : seg ? static_cast<size_t>(kstride) * W : static_cast<size_t>(kstride) * 2 + nodes + 2 * W + 2;
+    const size_t per_warp = (rows + static_cast<size_t>(epi) * 2) * kTile * sizeof(float);
     while (wpb > 1 && per_warp * wpb > 200 * 1024) wpb >>= 1;
     const size_t smem = per_warp * wpb;
-    SweepArgs args{b.insts, b.tile_prefix[cls], b.tile_first[cls], b.n_inst, total, kstride, mm_flags, epi};
+    SweepArgs args{b.insts, b.tile_prefix[cls], b.tile_first[cls], b.n_inst, total, kstride, nodes, mm_flags, epi};
     const int blocks = blocks_for(total, wpb, cfg.max_waves > 0 ? cfg.max_waves * cfg.num_sms * (2048 / (32 * wpb)) : (1 << 30));
     const bool timed = cfg.prof && cfg.prof->on && (mode == kFwdUpdate || mode == kBwdUpdate);
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;

@@ -66,6 +66,7 @@ struct DevBatch {
     int32_t* tile_first[kNumClasses] = {};   // [n_inst] first tile of class c in the instance
     int32_t tiles_total[kNumClasses] = {};
     int32_t kmax[kNumClasses] = {};
+    int32_t nodes_max[kNumClasses] = {};
     int32_t* var_prefix = nullptr;           // [n_inst + 1]
     int32_t vars_total = 0;
     int32_t* tile_all_prefix = nullptr;      // [n_inst + 1] all tiles of every class

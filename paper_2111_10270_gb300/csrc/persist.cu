@@ -93,7 +93,7 @@ __device__ __forceinline__ void sweep_pass(const SweepArgs (&c)[2], int n_reg, i
     for (int g = gw; g < n_seg + n_reg; g += nw) {
         const int gn = g + nw;
         if (g < n_seg) seg_tile<2, MODE>(c[kSegClass], g, gn < n_seg ? gn : n_seg, wsm, lane);
-        else sweep_tile<2, true, MODE>(c[kRegClass], g - n_seg, gn - n_seg, wsm, lane);
+        else reg_tile<2, MODE>(c[kRegClass], g - n_seg, gn - n_seg, wsm, lane);
     }
 }
 
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kPersistThreads, 2) persist_iterations_kernel(
 SweepArgs class_args(const DevBatch& b, int cls) {
     const int kstride = class_is_seg(cls) ? (b.kmax[cls] + kRegK - 1) / kRegK : 0;
     const int epi = b.has_local[cls] ? std::min(b.kmax[cls], kEpiMaxK) : 0;
-    return SweepArgs{b.insts, b.tile_prefix[cls], b.tile_first[cls], b.n_inst, b.tiles_total[cls], kstride, 0, epi};
+    return SweepArgs{b.insts, b.tile_prefix[cls], b.tile_first[cls], b.n_inst, b.tiles_total[cls], kstride, 0, 0, epi};
 }
 
 }  // namespace
@@ -163,7 +163,7 @@ bool persist_supported(const DevBatch& b) {
 }
 
 size_t persist_smem_bytes(const DevBatch& b) {
-    const int64_t wf = std::max<int64_t>(static_cast<int64_t>(sweep_warp_floats<2, true>(class_args(b, kRegClass))),
+    const int64_t wf = std::max<int64_t>(static_cast<int64_t>(reg_warp_floats(class_args(b, kRegClass))),
                                           static_cast<int64_t>(seg_warp_floats<2>(class_args(b, kSegClass))));
     return static_cast<size_t>(wf) * sizeof(float) * (kPersistThreads / 32);
 }

@@ -77,25 +77,13 @@ __device__ __forceinline__ void push(float (&x)[W], uint32_t code, float val) {
         if (code == static_cast<uint32_t>(w)) x[w] = fminf(x[w], val);
 }
 
-// per-layer state of one BDD: registers for short rows, shared memory otherwise
-template <int W, bool REG>
-struct Store;
-
+// per-layer state of one BDD of a short narrow row
 template <int W>
-struct Store<W, true> {
+struct Store {
     float lam[kRegK], tb[kRegK], sp[kRegK][W];
     __device__ __forceinline__ float& L(int t) { return lam[t]; }
     __device__ __forceinline__ float& T(int t) { return tb[t]; }
     __device__ __forceinline__ float& S(int t, int v) { return sp[t][v]; }
-};
-
-template <int W>
-struct Store<W, false> {
-    float* base;  // this lane's column of the warp's region
-    int stride;
-    __device__ __forceinline__ float& L(int t) { return base[t * kTile]; }
-    __device__ __forceinline__ float& T(int t) { return base[(stride + t) * kTile]; }
-    __device__ __forceinline__ float& S(int t, int v) { return base[(2 * stride + t * W + v) * kTile]; }
 };
 
 
@@ -142,24 +130,40 @@ __device__ __forceinline__ void prefetch_tile(const SweepArgs& a, int g, int lan
     }
 }
 
-// Loops over layers.  With REG the trip count is the constant kRegK and the
-// loops unroll completely, so every index into Store is a compile-time
-// constant and the arrays stay in registers.
-#define FD_UP(t) _Pragma("unroll") for (int t = 0; t < (REG ? kRegK : k); ++t)
+// Loops over the layers of a register-held BDD.  The trip count is the
+// constant kRegK and the loops unroll completely, so every index into Store
+// is a compile-time constant and the arrays stay in registers.
+#define FD_UP(t) _Pragma("unroll") for (int t = 0; t < kRegK; ++t)
 #define FD_DOWN(t, tt) \
-    _Pragma("unroll") for (int tt = 0; tt < (REG ? kRegK : k); ++tt) \
-        if (const int t = (REG ? kRegK : k) - 1 - tt; t < k)
+    _Pragma("unroll") for (int tt = 0; tt < kRegK; ++tt) \
+        if (const int t = kRegK - 1 - tt; t < k)
 
-// shared-memory floats one warp of sweep_tile uses
-template <int W, bool REG>
-__host__ __device__ __forceinline__ size_t sweep_warp_floats(const SweepArgs& a) {
-    return (REG ? 0 : static_cast<size_t>(a.kstride) * kTile * (2 + W)) + static_cast<size_t>(a.epi) * kTile * 2;
+// compensated FP32 butterfly of the lanes' shares of the bound (all lanes end equal)
+__device__ __forceinline__ float2 tile_bound(float s) {
+    float comp = 0.f;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const float o = __shfl_xor_sync(kFull, s, off);
+        const float oc = __shfl_xor_sync(kFull, comp, off);
+        const float sum = s + o;
+        const float bp = sum - s;
+        const float err = (s - (sum - bp)) + (o - bp);
+        s = sum;
+        comp = comp + oc + err;
+    }
+    return make_float2(s, comp);
 }
 
-// One tile g of a class (lane = BDD), the warp's shared memory at wsm; the
+// shared-memory floats one warp of reg_tile uses
+__host__ __device__ __forceinline__ size_t reg_warp_floats(const SweepArgs& a) {
+    return static_cast<size_t>(a.epi) * kTile * 2;
+}
+
+// Short rows (at most kRegK layers) of narrow BDDs (W <= kRegW): everything in
+// registers.  One tile g of a class (lane = BDD), the warp's shared memory at wsm; the
 // tile this warp visits next (g_next, if below a.total) is prefetched into L2.
-template <int W, bool REG, int MODE>
-__device__ __forceinline__ void sweep_tile(const SweepArgs& a, int g, int g_next, float* wsm, int lane) {
+template <int W, int MODE>
+__device__ __forceinline__ void reg_tile(const SweepArgs& a, int g, int g_next, float* wsm, int lane) {
     {
         prefetch_tile(a, g_next, lane);
         const int ii = find_inst(a.prefix, a.n_inst, g);
@@ -177,13 +181,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, int g, int g_next
         float* __restrict__ lam = I->lam;
         const bool need_t = (MODE == kFwdUpdate || MODE == kBwdUpdate) || (a.flags & kMMAddT);
 
-        Store<W, REG> S;
-        // per-warp shared memory: [Store arrays (shared-memory variants)] [staging for tile-local sums]
-        if constexpr (!REG) {
-            S.base = wsm + lane;
-            S.stride = a.kstride;
-        }
-        float* ep_lam = wsm + (REG ? 0 : static_cast<size_t>(a.kstride) * kTile * (2 + W));
+        Store<W> S;
+        float* ep_lam = wsm;
         int* ep_var = reinterpret_cast<int*>(ep_lam + static_cast<size_t>(a.epi) * kTile);
         const bool local = (MODE == kFwdUpdate || MODE == kBwdUpdate) && a.epi > 0 && tile.pattern >= 0;
 
@@ -237,7 +236,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, int g, int g_next
                 if (t >= k) break;
                 uint32_t c[W];
                 load_codes<W>(tpl + t * W, c);
-                const int tn = REG ? ((t + 1 < kRegK) ? t + 1 : t) : ((t + 1 < k) ? t + 1 : t);
+                const int tn = (t + 1 < kRegK) ? t + 1 : t;
                 float b[W];
 #pragma unroll
                 for (int v = 0; v < W; ++v) b[v] = S.S(tn, v);  // unused on the last layer (terminal codes)
@@ -362,6 +361,223 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, int g, int g_next
     }
 }
 
+// Wide BDDs (W > kRegW): per-layer state in shared memory, one column per lane
+// (so no bank conflicts), rows of 32 floats: the multipliers and terms of
+// every layer, one row per node for the stored labels (a.nodes: most nodes of
+// a shape of the launch), two layers of running labels and two constant rows
+// for the terminals.  A layer's nodes are visited one by one up to the number
+// it has, and a successor's label is read from the row its code names, the
+// same for the whole warp.  Holding all W labels in registers and selecting
+// among them for every arc took some 500 selects per layer at W = 16 whatever
+// its nodes (99 us a sweep of 368 tiles of at most 12 layers).
+// shared-memory floats one warp of wide_tile uses
+template <int W>
+__host__ __device__ __forceinline__ size_t wide_warp_floats(const SweepArgs& a) {
+    return (static_cast<size_t>(a.kstride) * 2 + a.nodes + 2 * W + 2) * kTile + static_cast<size_t>(a.epi) * kTile * 2;
+}
+
+template <int W, int MODE>
+__device__ __forceinline__ void wide_tile(const SweepArgs& a, int g, int g_next, float* wsm, int lane) {
+    constexpr bool update = MODE == kFwdUpdate || MODE == kBwdUpdate;
+    constexpr bool asc = MODE != kBwdUpdate;  // labels SP(., TOP) first, then the layers in ascending order
+    prefetch_tile(a, g_next, lane);
+    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const InstDev* __restrict__ I = a.insts + ii;
+    if (update && FDOG_INACTIVE(I->ctl)) return;
+    const int ti = __ldg(a.first + ii) + (g - __ldg(a.prefix + ii));
+    const TileDev tile = I->tiles[ti];
+    const ShapeDev sh = I->shapes[tile.shape];
+    const int k = sh.k;
+    const uint16_t* __restrict__ tpl = I->tpl + sh.tpl_off;
+    const bool valid = lane < tile.n_valid;
+    const float omega = I->omega;
+    const size_t base = static_cast<size_t>(tile.slot_base) + lane;
+    float* __restrict__ lam = I->lam;
+    const bool local = update && a.epi > 0 && tile.pattern >= 0;
+
+    float* Lr = wsm + lane;                                   // multipliers, row t
+    float* Tr = Lr + static_cast<size_t>(a.kstride) * kTile;  // terms, row t
+    float* X = Tr + static_cast<size_t>(a.kstride) * kTile;   // TOP (0), BOT (inf)
+    float* R0 = X + 2 * kTile;                                // running labels of two neighbouring layers
+    float* S = R0 + 2 * W * kTile;                            // stored labels, layer after layer as they are formed
+    float* ep_lam = wsm + (static_cast<size_t>(a.kstride) * 2 + a.nodes + 2 * W + 2) * kTile;
+    int* ep_var = reinterpret_cast<int*>(ep_lam + static_cast<size_t>(a.epi) * kTile);
+
+    // codes of layer t: lane v < W holds node v's; padding nodes have code 0xFFFF
+    auto codes_of = [&](int t) -> uint32_t { return lane < W && t >= 0 && t < k ? __ldg(tpl + t * W + lane) : 0xFFFFu; };
+    auto count_of = [&](uint32_t c) { return __popc(__ballot_sync(kFull, c != 0xFFFFu)); };
+    // row of a successor: a node of the layer at `next`, or a terminal's constant row
+    auto row_of = [&](float* next, uint32_t code) -> float* {
+        return code < kCodeTop ? next + code * kTile : X + (code - kCodeTop) * kTile;
+    };
+
+    X[0] = 0.f;
+    X[kTile] = finf();
+#pragma unroll 4
+    for (int t = 0; t < k; ++t) {
+        const size_t p = base + static_cast<size_t>(t) * kTile;
+        Lr[t * kTile] = lam[p];
+        if (update) Tr[t * kTile] = __int_as_float(__ldcs(I->var + p));  // streamed once per pass
+    }
+    if constexpr (update) {
+        const float* Tv = I->T;
+        if (local)
+            for (int t = 0; t < k; ++t) ep_var[t * kTile + lane] = __float_as_int(Tr[t * kTile]);
+#pragma unroll 4
+        for (int t = 0; t < k; ++t) {
+            const int v = __float_as_int(Tr[t * kTile]);
+            Tr[t * kTile] = v >= 0 ? Tv[v] : 0.f;
+        }
+    }
+
+    // labels of the direction opposite to the pass, at the current multipliers.
+    // asc: SP(v, TOP), from the last layer (Alg. 4); each layer's rows follow the next layer's.
+    // else: SP(r, v), from the root (Alg. 3); each layer's rows follow the one before.
+    float* at = S;  // rows of the layer last completed
+    float term = 0.f;
+    {
+        uint32_t c = codes_of(asc ? k - 1 : 0);
+        int n = count_of(c);
+        if constexpr (asc) {
+            float* next = X;  // the last layer has terminal codes only
+            for (int t = k - 1; t >= 0; --t) {
+                const uint32_t cp = codes_of(t - 1);  // in flight while this layer is formed
+                const float lt = Lr[t * kTile];
+                for (int v = 0; v < n; ++v) {
+                    const uint32_t cv = __shfl_sync(kFull, c, v);
+                    at[v * kTile] = fminf(*row_of(next, cv & 0xFFu), *row_of(next, cv >> 8) + lt);
+                }
+                next = at;
+                at += n * kTile;
+                c = cp;
+                n = count_of(c);
+            }
+            at = next;  // layer 0
+            if constexpr (MODE == kEval) term = at[0];
+        } else {
+            at[0] = 0.f;
+            for (int t = 0; t + 1 < k; ++t) {
+                const uint32_t cn = codes_of(t + 1);
+                const int nn = count_of(cn);
+                float* next = at + n * kTile;
+                for (int v = 0; v < nn; ++v) next[v * kTile] = finf();
+                const float lt = Lr[t * kTile];
+                for (int v = 0; v < n; ++v) {
+                    const uint32_t cv = __shfl_sync(kFull, c, v);
+                    const uint32_t lo = cv & 0xFFu, hi = cv >> 8;
+                    const float f = at[v * kTile];
+                    if (lo < kCodeTop) next[lo * kTile] = fminf(next[lo * kTile], f);
+                    if (hi < kCodeTop) next[hi * kTile] = fminf(next[hi * kTile], f + lt);
+                }
+                at = next;
+                c = cn;
+                n = nn;
+            }
+        }
+    }
+
+    if constexpr (MODE == kFwdUpdate || MODE == kMinMarg) {
+        // ascending pass: SP(r, .) incrementally (Alg. 3) and Eq. 6 per layer
+        float* f = R0;
+        float* fn = R0 + W * kTile;
+        f[0] = 0.f;
+        float* __restrict__ mm0 = I->mm0;
+        float* __restrict__ mm1 = I->mm1;
+        uint32_t c = codes_of(0);
+        int n = count_of(c);
+        for (int t = 0; t < k; ++t) {
+            const uint32_t cn = codes_of(t + 1);
+            const int nn = count_of(cn);
+            float* next = at - nn * kTile;  // SP(., TOP) of layer t + 1
+            float m0 = finf(), m1 = finf();
+            for (int v = 0; v < n; ++v) {
+                const uint32_t cv = __shfl_sync(kFull, c, v);
+                const float fv = f[v * kTile];
+                m0 = fminf(m0, fv + *row_of(next, cv & 0xFFu));
+                m1 = fminf(m1, fv + *row_of(next, cv >> 8));
+            }
+            float lt = Lr[t * kTile];
+            m1 += lt;
+            if constexpr (MODE == kFwdUpdate) {
+                lt = fmaf(-omega, m1 - m0, lt) + Tr[t * kTile];  // Eq. 5
+                Lr[t * kTile] = lt;
+            } else if (valid) {
+                const size_t p = base + static_cast<size_t>(t) * kTile;
+                if (a.flags & kMMBoth) { mm0[p] = m0; mm1[p] = m1; }
+                else mm0[p] = m1 - m0;
+            }
+            for (int v = 0; v < nn; ++v) fn[v * kTile] = finf();
+            for (int v = 0; v < n; ++v) {
+                const uint32_t cv = __shfl_sync(kFull, c, v);
+                const uint32_t lo = cv & 0xFFu, hi = cv >> 8;
+                const float fv = f[v * kTile];
+                if (lo < kCodeTop) fn[lo * kTile] = fminf(fn[lo * kTile], fv);
+                if (hi < kCodeTop) fn[hi * kTile] = fminf(fn[hi * kTile], fv + lt);
+            }
+            float* h = f;
+            f = fn;
+            fn = h;
+            at = next;
+            c = cn;
+            n = nn;
+        }
+    }
+
+    if constexpr (MODE == kBwdUpdate) {
+        // descending pass: SP(., TOP) incrementally (Alg. 4) and Eq. 6 per layer
+        float* b = R0;
+        float* bn = R0 + W * kTile;
+        float negsum = 0.f;
+        uint32_t c = codes_of(k - 1);
+        int n = count_of(c);
+        for (int t = k - 1; t >= 0; --t) {
+            const uint32_t cp = codes_of(t - 1);
+            float m0 = finf(), m1 = finf();
+            for (int v = 0; v < n; ++v) {
+                const uint32_t cv = __shfl_sync(kFull, c, v);
+                const float fv = at[v * kTile];
+                m0 = fminf(m0, fv + *row_of(b, cv & 0xFFu));
+                m1 = fminf(m1, fv + *row_of(b, cv >> 8));
+            }
+            float lt = Lr[t * kTile];
+            m1 += lt;
+            const float d = m1 - m0;
+            lt = fmaf(-omega, d, lt) + Tr[t * kTile];  // Eq. 5
+            Lr[t * kTile] = lt;
+            negsum += fmaxf(-d, 0.f);
+            for (int v = 0; v < n; ++v) {
+                const uint32_t cv = __shfl_sync(kFull, c, v);
+                bn[v * kTile] = fminf(*row_of(b, cv & 0xFFu), *row_of(b, cv >> 8) + lt);
+            }
+            float* h = b;
+            b = bn;
+            bn = h;
+            c = cp;
+            n = count_of(c);
+            at -= n * kTile;
+        }
+        term = fmaf(-omega, negsum, b[0]);
+    }
+
+    if constexpr (update) {
+#pragma unroll 4
+        for (int t = 0; t < k; ++t) {
+            if (valid) lam[base + static_cast<size_t>(t) * kTile] = Lr[t * kTile];
+        }
+        if (local) {
+            for (int t = 0; t < k; ++t) ep_lam[t * kTile + lane] = Lr[t * kTile];
+            __syncwarp();
+            tile_local_sums(I, tile.pattern, ep_lam, ep_var, lane);
+            __syncwarp();
+        }
+    }
+    if constexpr (MODE == kBwdUpdate || MODE == kEval) {
+        const float2 p = tile_bound(valid ? term : 0.f);
+        if (lane == 0) I->tile_lb[ti] = p;
+    }
+}
+
+// the register and the shared-memory tiles behind one name
 template <int W, bool REG, int MODE>
 __global__ void __launch_bounds__(256) sweep_kernel(SweepArgs a) {
     extern __shared__ float smem[];
@@ -370,9 +586,11 @@ __global__ void __launch_bounds__(256) sweep_kernel(SweepArgs a) {
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const int wpb = blockDim.x >> 5;
-    float* wsm = smem + static_cast<size_t>(wib) * sweep_warp_floats<W, REG>(a);
-    for (int g = blockIdx.x * wpb + wib; g < a.total; g += gridDim.x * wpb)
-        sweep_tile<W, REG, MODE>(a, g, g + gridDim.x * wpb, wsm, lane);
+    float* wsm = smem + static_cast<size_t>(wib) * (REG ? reg_warp_floats(a) : wide_warp_floats<W>(a));
+    for (int g = blockIdx.x * wpb + wib; g < a.total; g += gridDim.x * wpb) {
+        if constexpr (REG) reg_tile<W, MODE>(a, g, g + gridDim.x * wpb, wsm, lane);
+        else wide_tile<W, MODE>(a, g, g + gridDim.x * wpb, wsm, lane);
+    }
 }
 
 

@@ -1,0 +1,74 @@
+"""Sweep kernels at the edges of their tiles: every kernel class (short, long
+and wide rows), tiles of 1, 31, 32 and 33 BDDs, rows that end on and beside the
+segment and register limits, against the FP64 oracle with the tolerances of the
+other parity tests."""
+import numpy as np
+import pytest
+
+import ilpgen
+from parity_util import MM_RTOL, lb_close, rel_err, slot_order
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2111_10270_gb300 import build as b
+
+    b.build()
+    import paper_2111_10270_gb300 as P
+
+    return P
+
+
+def rows_ilp(coef, sense, rhs, count, seed, shared):
+    """`count` rows of one pattern.  With `shared`, neighbouring rows have half of their variables in common (all
+    copies of those in one tile, or split over two); the other variables lie in one row each."""
+    k = len(coef)
+    step = max(1, k // 2) if shared else k
+    rng = np.random.default_rng(seed)
+    n = step * (count - 1) + k
+    col = (np.arange(count)[:, None] * step + np.arange(k)).reshape(-1)
+    return ilpgen.ILP(n, rng.standard_normal(n), np.arange(count + 1, dtype=np.int64) * k, col.astype(np.int32),
+                      np.tile(np.asarray(coef, np.int32), count), np.full(count, sense, np.int8),
+                      np.full(count, rhs, np.int64), name="rows")
+
+
+PATTERNS = {
+    # short rows of width 2: at most one, flow, product, marginalisation, at least one
+    "amo2": ([1, 1], -1, 1), "amo8": ([1] * 8, -1, 1), "flow5": ([-1, 1, 1, 1, 1], -1, 0),
+    "product": ([1, 1, -1], -1, 1), "marg6": ([-1, 1, 1, 1, 1, 1], 0, 0), "cover7": ([1] * 7, 1, 1),
+    # short rows of width up to 4
+    "card6": ([1] * 6, -1, 3), "knap7": ([2, 1, 1, 2, 1, 1, 1], -1, 3), "exact5": ([1] * 5, 0, 2),
+    # long rows: on, one below and one above the segment length
+    "amo9": ([1] * 9, -1, 1), "flow16": ([-1] + [1] * 15, -1, 0), "amo17": ([1] * 17, 0, 1),
+    "flow24": ([-1] + [1] * 23, -1, 0), "cover25": ([1] * 25, 1, 1), "card16": ([1] * 16, -1, 2),
+    "card33": ([1] * 33, -1, 3), "mixed12": ([1, -1] * 6, -1, 1),
+    # wide rows
+    "knap4": ([3, 5, 7, 6], -1, 11), "knap8": ([3, 1, 2, 3, 1, 2, 3, 2], -1, 8), "knap9": ([1, 2, 3] * 3, -1, 9),
+    "card16w": ([1] * 16, -1, 7), "knap12": ([3, 2, 1, 3, 2, 3, 1, 2, 3, 1, 2, 3], 1, 13),
+    "exact40": ([1, 2] * 20, 0, 7),
+}
+
+
+@pytest.mark.parametrize("count", [1, 31, 32, 33])
+@pytest.mark.parametrize("shared", [False, True], ids=["apart", "shared"])
+@pytest.mark.parametrize("name", sorted(PATTERNS))
+def test_tile_edges(P, oracle_mod, name, shared, count):
+    coef, sense, rhs = PATTERNS[name]
+    g = rows_ilp(coef, sense, rhs, count, len(name) * 100 + count, shared)
+    inst = P.Instance.from_ilp(g, P.capi.default_params(tol=0.0, jit=-1)).build(0)
+    orc = oracle_mod.Problem.from_ilp(g)
+    for _ in range(6):
+        done, lb = inst.iterate(1)
+        olb = orc.iterate(1)[0]
+        assert done == 1 and lb_close(lb, olb, scale=np.abs(orc.energies()).sum()), (lb, olb)
+    var, row, m0, m1 = inst.min_marginals()
+    perm = slot_order(orc, var, row)
+    om0, om1 = orc.min_marginals()
+    assert rel_err(m0[perm], om0).max() <= MM_RTOL and rel_err(m1[perm], om1).max() <= MM_RTOL
+    _, fea = inst.lower_bound()
+    assert lb_close(fea, orc.lower_bounds()[1], scale=np.abs(orc.energies()).sum())
