@@ -66,7 +66,7 @@ static std::vector<Item> arena_items(const fdog_instance* inst, DevArrays& a) {
         {reinterpret_cast<void**>(&a.ctl), sizeof(InstCtl)},
         {reinterpret_cast<void**>(&a.tiles), sizeof(TileDev) * sz(nt)},
         {reinterpret_cast<void**>(&a.shapes), sizeof(ShapeDev) * sz(static_cast<int64_t>(d.shape_dev.size()))},
-        {reinterpret_cast<void**>(&a.tpl), sizeof(uint16_t) * std::max<size_t>(d.tpl.size(), 8)},
+        {reinterpret_cast<void**>(&a.tpl), sizeof(uint16_t) * (d.tpl.size() + kTplPad)},
         {reinterpret_cast<void**>(&a.lam), sizeof(float) * sz(S)},
         {reinterpret_cast<void**>(&a.var), sizeof(int32_t) * sz(S)},
         {reinterpret_cast<void**>(&a.mm0), sizeof(float) * sz(S)},

@@ -28,6 +28,11 @@ constexpr int kTile = 32;
 constexpr uint8_t kCodeTop = 0xFE;
 constexpr uint8_t kCodeBot = 0xFF;
 
+// The sweeps read the codes of kRegK layers at once, so up to kRegK layers of
+// kRegW codes beyond a shape's last one: the device array of templates is
+// this much longer than its contents.
+constexpr int kTplPad = 64;
+
 // Kernel classes: maximum layer width W of the shape (register arrays of W
 // shortest-path labels per layer) and whether all per-layer state fits in
 // registers (W <= kRegW and k <= kRegK) or lives in shared memory.
@@ -167,7 +172,7 @@ struct SweepArgs {
     int32_t total;
     int32_t kstride;        // wide BDDs: longest row; long rows: most checkpoints of a row
     int32_t nodes;          // wide BDDs: most nodes of a shape
-    int32_t flags;          // evaluate at lambda + T (1) | write m0 and m1 (2)
+    int32_t flags;          // min-marginals: write m0 and m1 (2)
     int32_t epi;            // update passes: layer stride of the per-warp staging for tile-local
                             // deferred sums (0: no tile of this launch has local variables)
 };

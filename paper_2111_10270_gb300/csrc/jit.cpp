@@ -135,16 +135,11 @@ void emit_shape(std::ostringstream& o, const HostShape& s, int id, int mode) {
     for (int t = 0; t < k; ++t) o << "  float " << nm("l", t) << " = 0.f, " << nm("u", t) << " = 0.f;\n";
     o << "  if (valid) {\n";
     for (int t = 0; t < k; ++t) o << "    " << nm("l", t) << " = lam[base + " << 32 * t << "];\n";
-    const char* need_u = mode <= 1 ? "true" : "(flags & 1)";
-    o << "    if (" << need_u << ") {\n";
-    for (int t = 0; t < k; ++t) {
-        o << "      { const int v = __ldcs(I->var + base + " << 32 * t << "); " << nm("u", t) << " = I->T[v];";
-        if (mode <= 1) o << " if (local) ep_var[" << 32 * t << "] = v;";
-        o << " }\n";
-    }
-    if (mode >= 2)
-        for (int t = 0; t < k; ++t) o << "      " << nm("l", t) << " += " << nm("u", t) << ";\n";
-    o << "    }\n  }\n";
+    if (mode <= 1)
+        for (int t = 0; t < k; ++t)
+            o << "    { const int v = __ldcs(I->var + base + " << 32 * t << "); " << nm("u", t)
+              << " = I->T[v]; if (local) ep_var[" << 32 * t << "] = v; }\n";
+    o << "  }\n";
 
     // b<t>_<v> = SP(node, TOP) at the current multipliers for layers [from, k)
     auto emit_backward_labels = [&](int from) {

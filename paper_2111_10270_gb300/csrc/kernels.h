@@ -17,8 +17,7 @@ enum SweepMode : int {
     kEval = 3,       // energies E^j only, no update
 };
 
-// kMinMarg / kEval flags
-constexpr int kMMAddT = 1;   // evaluate at lambda + T (the add-back of Alg. 1)
+// kMinMarg flags
 constexpr int kMMBoth = 2;   // write m0 and m1 (else M = m1 - m0 into mm0)
 
 // lower-bound reduction target: the bound of an iteration into InstCtl::lb_staged (committed later);

@@ -77,15 +77,97 @@ __device__ __forceinline__ void push(float (&x)[W], uint32_t code, float val) {
         if (code == static_cast<uint32_t>(w)) x[w] = fminf(x[w], val);
 }
 
-// per-layer state of one BDD of a short narrow row
+// Codes of one layer, two arcs (lo | hi << 8) to a word.
 template <int W>
-struct Store {
-    float lam[kRegK], tb[kRegK], sp[kRegK][W];
-    __device__ __forceinline__ float& L(int t) { return lam[t]; }
-    __device__ __forceinline__ float& T(int t) { return tb[t]; }
-    __device__ __forceinline__ float& S(int t, int v) { return sp[t][v]; }
+struct LayerCodes {
+    uint32_t w[W / 2];
+    __device__ __forceinline__ uint32_t lo(int v) const { return (w[v / 2] >> (16 * (v % 2))) & 0xFFu; }
+    __device__ __forceinline__ uint32_t hi(int v) const { return (w[v / 2] >> (16 * (v % 2) + 8)) & 0xFFu; }
 };
 
+// Codes of the kRegK layers from layer t0 on (a multiple of kRegK), all loads
+// issued together: templates start on 16 bytes and a layer takes 2 W bytes.
+// Beyond the shape's last layer the words are whatever follows it in memory
+// (the template array has room for them) and are not used.
+template <int W>
+__device__ __forceinline__ void load_segment_codes(const uint16_t* __restrict__ tpl, int t0, LayerCodes<W> (&c)[kRegK]) {
+    const uint4* __restrict__ p = reinterpret_cast<const uint4*>(tpl + static_cast<size_t>(t0) * W);
+#pragma unroll
+    for (int q = 0; q < kRegK * W / 8; ++q) {
+        const uint4 u = __ldg(p + q);
+        const uint32_t x[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) c[(4 * q + j) / (W / 2)].w[(4 * q + j) % (W / 2)] = x[j];
+    }
+}
+
+// Inner layers of 0/1 rows have one of two width-2 structures, equal up to
+// the order of the nodes: one node that may still take a 1 (which leads to
+// the other) and one that may not.  Most layers of matching, flow and
+// marginalisation rows are these; they take a handful of instructions where
+// the general step selects every successor among four.  The code is the same
+// for the whole warp, so the choice costs one uniform branch.
+constexpr uint32_t kStepUp = 0xFF010100u;    // node 0: 0 -> 0, 1 -> 1; node 1: 0 -> 1, 1 -> BOT
+constexpr uint32_t kStepDown = 0x0001FF00u;  // node 0: 0 -> 0, 1 -> BOT; node 1: 0 -> 1, 1 -> 0
+
+// labels SP(v, TOP) of a layer from those of the next one (Alg. 4)
+template <int W>
+__device__ __forceinline__ void pull_labels(float (&x)[W], const LayerCodes<W>& c, float l) {
+    if (W == 2 && c.w[0] == kStepUp) {
+        x[0] = fminf(x[0], x[1] + l);
+    } else if (W == 2 && c.w[0] == kStepDown) {
+        x[1] = fminf(x[1], x[0] + l);
+    } else {
+        float cur[W];
+#pragma unroll
+        for (int v = 0; v < W; ++v) cur[v] = fminf(pick<W>(x, c.lo(v)), pick<W>(x, c.hi(v)) + l);
+#pragma unroll
+        for (int v = 0; v < W; ++v) x[v] = cur[v];
+    }
+}
+
+// labels SP(r, v) of the next layer from those of this one (Alg. 3)
+template <int W>
+__device__ __forceinline__ void push_labels(float (&x)[W], const LayerCodes<W>& c, float l) {
+    if (W == 2 && c.w[0] == kStepUp) {
+        x[1] = fminf(x[0] + l, x[1]);
+    } else if (W == 2 && c.w[0] == kStepDown) {
+        x[0] = fminf(x[0], x[1] + l);
+    } else {
+        float nx[W];
+#pragma unroll
+        for (int v = 0; v < W; ++v) nx[v] = finf();
+#pragma unroll
+        for (int v = 0; v < W; ++v) {
+            push<W>(nx, c.lo(v), x[v]);
+            push<W>(nx, c.hi(v), x[v] + l);
+        }
+#pragma unroll
+        for (int v = 0; v < W; ++v) x[v] = nx[v];
+    }
+}
+
+// Eq. 6 of a layer without the layer's own multiplier in m1: f its labels
+// SP(r, .), b the next layer's SP(., TOP)
+template <int W>
+__device__ __forceinline__ void layer_marginals(const float (&f)[W], const float (&b)[W], const LayerCodes<W>& c,
+                                                float& m0, float& m1) {
+    if (W == 2 && c.w[0] == kStepUp) {
+        m0 = fminf(f[0] + b[0], f[1] + b[1]);
+        m1 = f[0] + b[1];
+    } else if (W == 2 && c.w[0] == kStepDown) {
+        m0 = fminf(f[0] + b[0], f[1] + b[1]);
+        m1 = f[1] + b[0];
+    } else {
+        m0 = finf();
+        m1 = finf();
+#pragma unroll
+        for (int v = 0; v < W; ++v) {
+            m0 = fminf(m0, f[v] + pick<W>(b, c.lo(v)));
+            m1 = fminf(m1, f[v] + pick<W>(b, c.hi(v)));
+        }
+    }
+}
 
 // 1 / c rounded to FP32 for a copy count c <= 8 (constants folded at compile
 // time); the deferred term of a variable is (C_i - sum_j lambda^j_i) times it
@@ -131,12 +213,10 @@ __device__ __forceinline__ void prefetch_tile(const SweepArgs& a, int g, int lan
 }
 
 // Loops over the layers of a register-held BDD.  The trip count is the
-// constant kRegK and the loops unroll completely, so every index into Store
-// is a compile-time constant and the arrays stay in registers.
-#define FD_UP(t) _Pragma("unroll") for (int t = 0; t < kRegK; ++t)
-#define FD_DOWN(t, tt) \
-    _Pragma("unroll") for (int tt = 0; tt < kRegK; ++tt) \
-        if (const int t = kRegK - 1 - tt; t < k)
+// constant kRegK and the loops unroll completely, so every index is a
+// compile-time constant and the arrays stay in registers.
+#define FD_UP(t) _Pragma("unroll") for (int t = 0; t < kRegK; ++t) if (t < k)
+#define FD_DOWN(t) _Pragma("unroll") for (int t = kRegK - 1; t >= 0; --t) if (t < k)
 
 // compensated FP32 butterfly of the lanes' shares of the bound (all lanes end equal)
 __device__ __forceinline__ float2 tile_bound(float s) {
@@ -160,204 +240,124 @@ __host__ __device__ __forceinline__ size_t reg_warp_floats(const SweepArgs& a) {
 }
 
 // Short rows (at most kRegK layers) of narrow BDDs (W <= kRegW): everything in
-// registers.  One tile g of a class (lane = BDD), the warp's shared memory at wsm; the
-// tile this warp visits next (g_next, if below a.total) is prefetched into L2.
+// registers.  One tile g of a class (lane = BDD), the warp's shared memory at
+// wsm; the tile this warp visits next (g_next, if below a.total) is
+// prefetched into L2.  A lone instance has about one tile per warp, so the
+// kernel's time is its chain of dependent loads: the codes of all layers, the
+// multipliers and the variable ids are each loaded at once, then all terms T
+// (interleaved layer by layer, every layer waited for its own id before the
+// next one's loads were issued).
 template <int W, int MODE>
 __device__ __forceinline__ void reg_tile(const SweepArgs& a, int g, int g_next, float* wsm, int lane) {
-    {
-        prefetch_tile(a, g_next, lane);
-        const int ii = find_inst(a.prefix, a.n_inst, g);
-        const InstDev* __restrict__ I = a.insts + ii;
-        if constexpr (MODE == kFwdUpdate || MODE == kBwdUpdate) {
-            if (FDOG_INACTIVE(I->ctl)) return;  // stopped, or out of iterations
+    constexpr bool update = MODE == kFwdUpdate || MODE == kBwdUpdate;
+    prefetch_tile(a, g_next, lane);
+    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const InstDev* __restrict__ I = a.insts + ii;
+    if (update && FDOG_INACTIVE(I->ctl)) return;  // stopped, or out of iterations
+    const int ti = __ldg(a.first + ii) + (g - __ldg(a.prefix + ii));
+    const TileDev tile = I->tiles[ti];
+    const ShapeDev sh = I->shapes[tile.shape];
+    const int k = sh.k;
+    const bool valid = lane < tile.n_valid;
+    const float omega = I->omega;
+    const size_t base = static_cast<size_t>(tile.slot_base) + lane;
+    float* __restrict__ lam = I->lam;
+    float* ep_lam = wsm;
+    int* ep_var = reinterpret_cast<int*>(ep_lam + static_cast<size_t>(a.epi) * kTile);
+    const bool local = update && a.epi > 0 && tile.pattern >= 0;
+
+    // padding lanes hold multiplier 0 and variable -1
+    LayerCodes<W> c[kRegK];
+    load_segment_codes<W>(I->tpl + sh.tpl_off, 0, c);
+    float L[kRegK], T[kRegK], S[kRegK][W];
+    int V[kRegK];
+    FD_UP(t) L[t] = lam[base + static_cast<size_t>(t) * kTile];
+    if constexpr (update) {
+        FD_UP(t) V[t] = __ldcs(I->var + base + static_cast<size_t>(t) * kTile);  // streamed once per pass
+        const float* Tv = I->T;
+        FD_UP(t) T[t] = V[t] >= 0 ? Tv[V[t]] : 0.f;
+        if (local) {
+            FD_UP(t) ep_var[t * kTile + lane] = V[t];
         }
-        const TileDev tile = I->tiles[__ldg(a.first + ii) + (g - __ldg(a.prefix + ii))];
-        const ShapeDev sh = I->shapes[tile.shape];
-        const int k = sh.k;
-        const uint16_t* __restrict__ tpl = I->tpl + sh.tpl_off;
-        const bool valid = lane < tile.n_valid;
-        const float omega = I->omega;
-        const size_t base = static_cast<size_t>(tile.slot_base) + lane;
-        float* __restrict__ lam = I->lam;
-        const bool need_t = (MODE == kFwdUpdate || MODE == kBwdUpdate) || (a.flags & kMMAddT);
+    }
 
-        Store<W> S;
-        float* ep_lam = wsm;
-        int* ep_var = reinterpret_cast<int*>(ep_lam + static_cast<size_t>(a.epi) * kTile);
-        const bool local = (MODE == kFwdUpdate || MODE == kBwdUpdate) && a.epi > 0 && tile.pattern >= 0;
-
-        // multipliers and deferred terms of every layer (coalesced per layer)
+    float term = 0.f;  // this BDD's share of the lower bound
+    float x[W];        // the running labels
+    if constexpr (MODE == kFwdUpdate || MODE == kMinMarg || MODE == kEval) {
+        // SP(v, TOP) of every node at the current multipliers (Alg. 4 without updates);
+        // S[t] the labels of layer t + 1 (the last layer's arcs lead to terminals: unused)
+#pragma unroll
+        for (int v = 0; v < W; ++v) x[v] = finf();
+        FD_DOWN(t) {
+#pragma unroll
+            for (int v = 0; v < W; ++v) S[t][v] = x[v];
+            pull_labels<W>(x, c[t], L[t]);
+        }
+        if constexpr (MODE == kEval) term = x[0];
+    } else {
+        // SP(r, v) of every node at the current multipliers (Alg. 3 without updates)
+#pragma unroll
+        for (int v = 0; v < W; ++v) x[v] = v == 0 ? 0.f : finf();
         FD_UP(t) {
-            if (t >= k) break;
-            float l = 0.f, tb = 0.f;
-            if (valid) {
-                l = lam[base + static_cast<size_t>(t) * kTile];
-                if (need_t) {
-                    const int v = __ldcs(I->var + base + static_cast<size_t>(t) * kTile);  // streamed once per pass
-                    tb = I->T[v];
-                    if (local) ep_var[t * kTile + lane] = v;
-                }
-            }
-            if constexpr (MODE == kMinMarg || MODE == kEval) {
-                if (a.flags & kMMAddT) l += tb;
-            }
-            S.L(t) = l;
-            S.T(t) = tb;
+#pragma unroll
+            for (int v = 0; v < W; ++v) S[t][v] = x[v];
+            push_labels<W>(x, c[t], L[t]);
         }
+    }
 
-        float term = 0.f;  // this BDD's share of the lower bound
-        if constexpr (MODE == kFwdUpdate || MODE == kMinMarg || MODE == kEval) {
-            // SP(v, TOP) of every node at the current multipliers (Alg. 4 without updates)
-            float nx[W];
+    if constexpr (MODE == kFwdUpdate || MODE == kMinMarg) {
+        // ascending pass: SP(r, .) incrementally (Alg. 3) and Eq. 6 per layer
 #pragma unroll
-            for (int v = 0; v < W; ++v) nx[v] = finf();
-            FD_DOWN(t, tt) {
-                uint32_t c[W];
-                load_codes<W>(tpl + t * W, c);
-                const float lt = S.L(t);
-                float cur[W];
-#pragma unroll
-                for (int v = 0; v < W; ++v) cur[v] = fminf(pick<W>(nx, c[v] & 0xFFu), pick<W>(nx, c[v] >> 8) + lt);
-#pragma unroll
-                for (int v = 0; v < W; ++v) { S.S(t, v) = cur[v]; nx[v] = cur[v]; }
+        for (int v = 0; v < W; ++v) x[v] = v == 0 ? 0.f : finf();
+        float* __restrict__ mm0 = I->mm0;
+        float* __restrict__ mm1 = I->mm1;
+        FD_UP(t) {
+            float m0, m1;
+            layer_marginals<W>(x, S[t], c[t], m0, m1);
+            m1 += L[t];
+            if constexpr (MODE == kFwdUpdate) {
+                L[t] = fmaf(-omega, m1 - m0, L[t]) + T[t];  // Eq. 5
+            } else if (valid) {
+                const size_t p = base + static_cast<size_t>(t) * kTile;
+                if (a.flags & kMMBoth) { mm0[p] = m0; mm1[p] = m1; }
+                else mm0[p] = m1 - m0;
             }
-            if constexpr (MODE == kEval) term = nx[0];
+            push_labels<W>(x, c[t], L[t]);
         }
+    }
 
-        if constexpr (MODE == kFwdUpdate || MODE == kMinMarg) {
-            // ascending pass: SP(r, .) incrementally (Alg. 3) and Eq. 6 per layer
-            float f[W];
+    if constexpr (MODE == kBwdUpdate) {
+        // descending pass: SP(., TOP) incrementally (Alg. 4) and Eq. 6 per layer
 #pragma unroll
-            for (int v = 0; v < W; ++v) f[v] = v == 0 ? 0.f : finf();
-            float negsum = 0.f, E = finf();
-            float* __restrict__ mm0 = I->mm0;
-            float* __restrict__ mm1 = I->mm1;
-            FD_UP(t) {
-                if (t >= k) break;
-                uint32_t c[W];
-                load_codes<W>(tpl + t * W, c);
-                const int tn = (t + 1 < kRegK) ? t + 1 : t;
-                float b[W];
-#pragma unroll
-                for (int v = 0; v < W; ++v) b[v] = S.S(tn, v);  // unused on the last layer (terminal codes)
-                float m0 = finf(), m1 = finf();
-#pragma unroll
-                for (int v = 0; v < W; ++v) {
-                    m0 = fminf(m0, f[v] + pick<W>(b, c[v] & 0xFFu));
-                    m1 = fminf(m1, f[v] + pick<W>(b, c[v] >> 8));
-                }
-                const float lt = S.L(t);
-                m1 += lt;
-                float lt_new = lt;
-                if constexpr (MODE == kFwdUpdate) {
-                    const float d = m1 - m0;
-                    lt_new = fmaf(-omega, d, lt) + S.T(t);  // Eq. 5
-                    S.L(t) = lt_new;
-                    negsum += fmaxf(-d, 0.f);
-                } else {
-                    if (valid) {
-                        const size_t p = base + static_cast<size_t>(t) * kTile;
-                        if (a.flags & kMMBoth) { mm0[p] = m0; mm1[p] = m1; }
-                        else mm0[p] = m1 - m0;
-                    }
-                }
-                float nf[W];
-#pragma unroll
-                for (int v = 0; v < W; ++v) nf[v] = finf();
-#pragma unroll
-                for (int v = 0; v < W; ++v) {
-                    const uint32_t lo = c[v] & 0xFFu, hi = c[v] >> 8;
-                    push<W>(nf, lo, f[v]);
-                    push<W>(nf, hi, f[v] + lt_new);
-                    E = fminf(E, lo == kCodeTop ? f[v] : finf());
-                    E = fminf(E, hi == kCodeTop ? f[v] + lt_new : finf());
-                }
-#pragma unroll
-                for (int v = 0; v < W; ++v) f[v] = nf[v];
-            }
-            term = fmaf(-omega, negsum, E);
+        for (int v = 0; v < W; ++v) x[v] = finf();
+        float negsum = 0.f;
+        FD_DOWN(t) {
+            float m0, m1;
+            layer_marginals<W>(S[t], x, c[t], m0, m1);
+            m1 += L[t];
+            const float d = m1 - m0;
+            L[t] = fmaf(-omega, d, L[t]) + T[t];  // Eq. 5
+            negsum += fmaxf(-d, 0.f);
+            pull_labels<W>(x, c[t], L[t]);
         }
+        term = fmaf(-omega, negsum, x[0]);
+    }
 
-        if constexpr (MODE == kBwdUpdate) {
-            // SP(r, v) of every node at the current multipliers (Alg. 3 without updates)
-            float f[W];
-#pragma unroll
-            for (int v = 0; v < W; ++v) f[v] = v == 0 ? 0.f : finf();
-            FD_UP(t) {
-                if (t >= k) break;
-                uint32_t c[W];
-                load_codes<W>(tpl + t * W, c);
-                const float lt = S.L(t);
-                float nf[W];
-#pragma unroll
-                for (int v = 0; v < W; ++v) { S.S(t, v) = f[v]; nf[v] = finf(); }
-#pragma unroll
-                for (int v = 0; v < W; ++v) {
-                    push<W>(nf, c[v] & 0xFFu, f[v]);
-                    push<W>(nf, c[v] >> 8, f[v] + lt);
-                }
-#pragma unroll
-                for (int v = 0; v < W; ++v) f[v] = nf[v];
-            }
-            // descending pass: SP(., TOP) incrementally (Alg. 4) and Eq. 6 per layer
-            float b[W];
-#pragma unroll
-            for (int v = 0; v < W; ++v) b[v] = finf();
-            float negsum = 0.f;
-            FD_DOWN(t, tt) {
-                uint32_t c[W];
-                load_codes<W>(tpl + t * W, c);
-                float m0 = finf(), m1 = finf();
-#pragma unroll
-                for (int v = 0; v < W; ++v) {
-                    const float fv = S.S(t, v);
-                    m0 = fminf(m0, fv + pick<W>(b, c[v] & 0xFFu));
-                    m1 = fminf(m1, fv + pick<W>(b, c[v] >> 8));
-                }
-                const float lt = S.L(t);
-                m1 += lt;
-                const float d = m1 - m0;
-                const float lt_new = fmaf(-omega, d, lt) + S.T(t);  // Eq. 5
-                S.L(t) = lt_new;
-                negsum += fmaxf(-d, 0.f);
-                float nb[W];
-#pragma unroll
-                for (int v = 0; v < W; ++v) nb[v] = fminf(pick<W>(b, c[v] & 0xFFu), pick<W>(b, c[v] >> 8) + lt_new);
-#pragma unroll
-                for (int v = 0; v < W; ++v) b[v] = nb[v];
-            }
-            term = fmaf(-omega, negsum, b[0]);
+    if constexpr (update) {
+        if (valid) {
+            FD_UP(t) lam[base + static_cast<size_t>(t) * kTile] = L[t];
         }
-
-        if constexpr (MODE == kFwdUpdate || MODE == kBwdUpdate) {
-            FD_UP(t) {
-                if (t >= k) break;
-                if (valid) lam[base + static_cast<size_t>(t) * kTile] = S.L(t);
-                if (local) ep_lam[t * kTile + lane] = S.L(t);
-            }
-            if (local) {
-                __syncwarp();
-                tile_local_sums(I, tile.pattern, ep_lam, ep_var, lane);
-                __syncwarp();
-            }
+        if (local) {
+            FD_UP(t) ep_lam[t * kTile + lane] = L[t];
+            __syncwarp();
+            tile_local_sums(I, tile.pattern, ep_lam, ep_var, lane);
+            __syncwarp();
         }
-
-        // per-tile partial of the bound: compensated FP32 butterfly (all lanes end equal); only the
-        // descending update pass and the energy sweep feed a bound reduction
-        if constexpr (MODE == kBwdUpdate || MODE == kEval) {  // the passes whose bound is reduced
-            float s = valid ? term : 0.f, comp = 0.f;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const float o = __shfl_xor_sync(kFull, s, off);
-                const float oc = __shfl_xor_sync(kFull, comp, off);
-                const float sum = s + o;
-                const float bp = sum - s;
-                const float err = (s - (sum - bp)) + (o - bp);
-                s = sum;
-                comp = comp + oc + err;
-            }
-            if (lane == 0) I->tile_lb[__ldg(a.first + ii) + (g - __ldg(a.prefix + ii))] = make_float2(s, comp);
-        }
+    }
+    // only the descending update pass and the energy sweep feed a bound reduction
+    if constexpr (MODE == kBwdUpdate || MODE == kEval) {
+        const float2 p = tile_bound(valid ? term : 0.f);
+        if (lane == 0) I->tile_lb[ti] = p;
     }
 }
 
@@ -598,12 +598,18 @@ __global__ void __launch_bounds__(256) sweep_kernel(SweepArgs a) {
 // every layer in shared memory would size each warp's region by the longest
 // row of the launch and starve the SM of warps, so the layers are processed
 // in segments of kRegK held in registers instead.  A first sweep over the
-// whole row keeps only the labels at segment starts (checkpoints, in shared
+// whole row keeps only the labels at segment ends (checkpoints, in shared
 // memory); the update sweep then visits the segments in its own direction,
-// reloads each one's multipliers and recomputes its labels from the next
+// reloads each one's multipliers and recomputes its labels from its
 // checkpoint.  Every label and update is formed by the same operations in the
-// same order as in sweep_kernel, so results are identical; the cost is one
-// extra label sweep over data the warp has just read.
+// same order as in reg_tile, so results are identical; the cost is one extra
+// label sweep over data the warp has just read.  As in reg_tile a segment's
+// codes, multipliers and ids are each loaded at once, and one segment (of the
+// ids: two) ahead of their use, so that no walk waits for memory in the middle.
+// A lone cell-tracking sequence (160 tiles) went from 25.7 and 20.7 us
+// (ascending, descending) to 20.1 and 16.4; what is left of a warp's 1,640
+// instructions is a chain: 10.5 cycles each, 4 of them memory, 2.8 the
+// latency of the operation before, 1.6 instruction fetch.
 // Shared memory per warp: a.kstride checkpoints x W labels x 32 lanes, then
 // the tile-local staging (a.epi layers).
 // shared-memory floats one warp of seg_tile uses
@@ -615,326 +621,196 @@ __host__ __device__ __forceinline__ size_t seg_warp_floats(const SweepArgs& a) {
 template <int W, int MODE>
 __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, float* wsm, int lane) {
     constexpr int C = kRegK;
-    float* cp = wsm + lane;  // checkpoint s, label v at cp[(s * W + v) * kTile]
+    constexpr bool update = MODE == kFwdUpdate || MODE == kBwdUpdate;
+    constexpr bool asc = MODE != kBwdUpdate;  // the update sweep's direction
+    float* cp = wsm + lane;  // checkpoint of segment s, label v at cp[(s * W + v) * kTile]
     float* ep_lam = wsm + static_cast<size_t>(a.kstride) * W * kTile;
     int* ep_var = reinterpret_cast<int*>(ep_lam + static_cast<size_t>(a.epi) * kTile);
-    {
-        prefetch_tile(a, g_next, lane);
-        const int ii = find_inst(a.prefix, a.n_inst, g);
-        const InstDev* __restrict__ I = a.insts + ii;
-        if constexpr (MODE == kFwdUpdate || MODE == kBwdUpdate) {
-            if (FDOG_INACTIVE(I->ctl)) return;
+    prefetch_tile(a, g_next, lane);
+    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const InstDev* __restrict__ I = a.insts + ii;
+    if (update && FDOG_INACTIVE(I->ctl)) return;
+    const int ti = __ldg(a.first + ii) + (g - __ldg(a.prefix + ii));
+    const TileDev tile = I->tiles[ti];
+    const ShapeDev sh = I->shapes[tile.shape];
+    const int k = sh.k;
+    const int nseg = (k + C - 1) / C;
+    const uint16_t* __restrict__ tpl = I->tpl + sh.tpl_off;
+    const bool valid = lane < tile.n_valid;
+    const float omega = I->omega;
+    const size_t base = static_cast<size_t>(tile.slot_base) + lane;
+    float* __restrict__ lam = I->lam;
+    const int32_t* __restrict__ varp = I->var;
+    const float* Tv = I->T;
+    const bool local = update && a.epi > 0 && tile.pattern >= 0;
+
+    // loads of one segment; padding lanes hold multiplier 0 and variable -1
+    auto fetch_lam = [&](int s, float (&L)[C]) {
+#pragma unroll
+        for (int j = 0; j < C; ++j)
+            if (s * C + j < k) L[j] = lam[base + static_cast<size_t>(s * C + j) * kTile];
+    };
+    auto fetch_var = [&](int s, int (&V)[C]) {
+#pragma unroll
+        for (int j = 0; j < C; ++j)
+            V[j] = s * C + j < k ? __ldcs(varp + base + static_cast<size_t>(s * C + j) * kTile) : -1;  // streamed
+    };
+    // terms of a segment's variables; ids staged for the tile-local sums
+    auto fetch_terms = [&](int s, const int (&V)[C], float (&T)[C]) {
+#pragma unroll
+        for (int j = 0; j < C; ++j) T[j] = V[j] >= 0 ? Tv[V[j]] : 0.f;
+        if (local) {
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+                if (s * C + j < k) ep_var[(s * C + j) * kTile + lane] = V[j];
         }
-        const TileDev tile = I->tiles[__ldg(a.first + ii) + (g - __ldg(a.prefix + ii))];
-        const ShapeDev sh = I->shapes[tile.shape];
-        const int k = sh.k;
-        const int nseg = (k + C - 1) / C;
-        const uint16_t* __restrict__ tpl = I->tpl + sh.tpl_off;
-        const bool valid = lane < tile.n_valid;
-        const float omega = I->omega;
-        const size_t base = static_cast<size_t>(tile.slot_base) + lane;
-        float* __restrict__ lam = I->lam;
-        const int32_t* __restrict__ varp = I->var;
-        const float* __restrict__ Tv = I->T;
-        constexpr bool update = MODE == kFwdUpdate || MODE == kBwdUpdate;
-        const bool need_t = update || (a.flags & kMMAddT);
-        const bool add_t = (MODE == kMinMarg || MODE == kEval) && (a.flags & kMMAddT);
-        const bool local = update && a.epi > 0 && tile.pattern >= 0;
+    };
+    // segments in the order of the update sweep are u = 0 .. nseg - 1, the label sweep visits them from the last
+    auto seg_of = [&](int u) { return asc ? u : nseg - 1 - u; };
 
-        // raw loads of one segment (multipliers, and variable ids if asked); independent of each other
-        auto fetch = [&](int s, float (&L)[C], int (&V)[C], bool with_var) {
-            const int t0 = s * C;
+    float x[W];
+    float L[C], T[C], Ln[C], Tn[C];
+    int V[C];
+    LayerCodes<W> c[C], cn[C];
+    // Label sweep: SP(v, TOP) over the whole row from its end (asc), SP(r, v) from its root (else); checkpoint of
+    // a segment: the labels it starts from.  The last segment visited is the update sweep's first, its
+    // multipliers and codes stay in L and c.
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                L[c] = 0.f;
-                V[c] = -1;
-                if (valid && t0 + c < k) {
-                    const size_t p = base + static_cast<size_t>(t0 + c) * kTile;
-                    L[c] = lam[p];
-                    if (with_var) V[c] = __ldcs(varp + p);  // streamed once per pass
-                }
-            }
-        };
-        // deferred terms of a fetched segment; with add_t the multipliers include them
-        auto terms = [&](float (&L)[C], const int (&V)[C], float (&Tt)[C]) {
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                Tt[c] = V[c] >= 0 ? Tv[V[c]] : 0.f;
-                if (add_t) L[c] += Tt[c];
-            }
-        };
-
-        float term = 0.f;
-        if constexpr (MODE == kFwdUpdate || MODE == kMinMarg || MODE == kEval) {
-            // SP(v, TOP) over the whole row, one segment at a time from the last;
-            // keep the labels at segment starts
-            float nx[W];
-#pragma unroll
-            for (int v = 0; v < W; ++v) nx[v] = finf();
-            for (int s = nseg - 1; s >= 0; --s) {
-                const int t0 = s * C;
-                const int kk = (k - t0 < C) ? k - t0 : C;
-                float L[C], Tt[C];
-                int V[C];
-                fetch(s, L, V, add_t);
-                if (add_t) terms(L, V, Tt);
-#pragma unroll
-                for (int cc = C - 1; cc >= 0; --cc) {
-                    if (cc < kk) {
-                        uint32_t c[W];
-                        load_codes<W>(tpl + (t0 + cc) * W, c);
-                        float cur[W];
-#pragma unroll
-                        for (int v = 0; v < W; ++v) cur[v] = fminf(pick<W>(nx, c[v] & 0xFFu), pick<W>(nx, c[v] >> 8) + L[cc]);
-#pragma unroll
-                        for (int v = 0; v < W; ++v) nx[v] = cur[v];
-                    }
-                }
-#pragma unroll
-                for (int v = 0; v < W; ++v) cp[(s * W + v) * kTile] = nx[v];
-            }
-            if constexpr (MODE == kEval) term = nx[0];
+    for (int v = 0; v < W; ++v) x[v] = !asc && v == 0 ? 0.f : finf();
+    fetch_lam(seg_of(nseg - 1), L);
+    load_segment_codes<W>(tpl, seg_of(nseg - 1) * C, c);
+    if constexpr (update) fetch_var(seg_of(0), V);
+    for (int u = nseg - 1; u >= 0; --u) {
+        const int s = seg_of(u);
+        const int kk = min(k - s * C, C);
+        if (u > 0) {  // in flight while this segment is swept
+            fetch_lam(seg_of(u - 1), Ln);
+            load_segment_codes<W>(tpl, seg_of(u - 1) * C, cn);
         }
-
-        if constexpr (MODE == kFwdUpdate || MODE == kMinMarg) {
-            float f[W];
 #pragma unroll
-            for (int v = 0; v < W; ++v) f[v] = v == 0 ? 0.f : finf();
-            float negsum = 0.f, E = finf();
-            float* __restrict__ mm0 = I->mm0;
-            float* __restrict__ mm1 = I->mm1;
-            float Ln[C];
-            int Vn[C];
-            fetch(0, Ln, Vn, need_t);
-            for (int s = 0; s < nseg; ++s) {
-                const int t0 = s * C;
-                const int kk = (k - t0 < C) ? k - t0 : C;
-                float L[C], Tt[C], Sg[C][W], nxt[W];
-                int V[C];
+        for (int v = 0; v < W; ++v) cp[(s * W + v) * kTile] = x[v];
+        if (u > 0 || MODE == kEval) {  // the first segment's own labels are formed by the update sweep
+            if constexpr (asc) {
 #pragma unroll
-                for (int c = 0; c < C; ++c) { L[c] = Ln[c]; V[c] = Vn[c]; }
-                if (s + 1 < nseg) fetch(s + 1, Ln, Vn, need_t);  // in flight while this segment is swept
-                terms(L, V, Tt);
-                if (local && valid) {
+                for (int j = C - 1; j >= 0; --j)
+                    if (j < kk) pull_labels<W>(x, c[j], L[j]);
+            } else {
 #pragma unroll
-                    for (int c = 0; c < C; ++c)
-                        if (c < kk) ep_var[(t0 + c) * kTile + lane] = V[c];
-                }
-                // labels of the segment's layers 1 .. kk-1, from the next checkpoint
-#pragma unroll
-                for (int v = 0; v < W; ++v) nxt[v] = (s + 1 < nseg) ? cp[((s + 1) * W + v) * kTile] : finf();
-                {
-                    float nx[W];
-#pragma unroll
-                    for (int v = 0; v < W; ++v) nx[v] = nxt[v];
-#pragma unroll
-                    for (int cc = C - 1; cc >= 1; --cc) {
-                        if (cc < kk) {
-                            uint32_t c[W];
-                            load_codes<W>(tpl + (t0 + cc) * W, c);
-                            float cur[W];
-#pragma unroll
-                            for (int v = 0; v < W; ++v)
-                                cur[v] = fminf(pick<W>(nx, c[v] & 0xFFu), pick<W>(nx, c[v] >> 8) + L[cc]);
-#pragma unroll
-                            for (int v = 0; v < W; ++v) { Sg[cc][v] = cur[v]; nx[v] = cur[v]; }
-                        }
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    if (c < kk) {
-                        const int t = t0 + c;
-                        uint32_t cd[W];
-                        load_codes<W>(tpl + t * W, cd);
-                        float b[W];
-#pragma unroll
-                        for (int v = 0; v < W; ++v) b[v] = (c + 1 < kk) ? Sg[(c + 1 < C) ? c + 1 : c][v] : nxt[v];
-                        float m0 = finf(), m1 = finf();
-#pragma unroll
-                        for (int v = 0; v < W; ++v) {
-                            m0 = fminf(m0, f[v] + pick<W>(b, cd[v] & 0xFFu));
-                            m1 = fminf(m1, f[v] + pick<W>(b, cd[v] >> 8));
-                        }
-                        const float lt = L[c];
-                        m1 += lt;
-                        float lt_new = lt;
-                        if constexpr (MODE == kFwdUpdate) {
-                            const float d = m1 - m0;
-                            lt_new = fmaf(-omega, d, lt) + Tt[c];  // Eq. 5
-                            L[c] = lt_new;
-                            negsum += fmaxf(-d, 0.f);
-                        } else {
-                            if (valid) {
-                                const size_t p = base + static_cast<size_t>(t) * kTile;
-                                if (a.flags & kMMBoth) { mm0[p] = m0; mm1[p] = m1; }
-                                else mm0[p] = m1 - m0;
-                            }
-                        }
-                        float nf[W];
-#pragma unroll
-                        for (int v = 0; v < W; ++v) nf[v] = finf();
-#pragma unroll
-                        for (int v = 0; v < W; ++v) {
-                            const uint32_t lo = cd[v] & 0xFFu, hi = cd[v] >> 8;
-                            push<W>(nf, lo, f[v]);
-                            push<W>(nf, hi, f[v] + lt_new);
-                            E = fminf(E, lo == kCodeTop ? f[v] : finf());
-                            E = fminf(E, hi == kCodeTop ? f[v] + lt_new : finf());
-                        }
-#pragma unroll
-                        for (int v = 0; v < W; ++v) f[v] = nf[v];
-                    }
-                }
-                if constexpr (MODE == kFwdUpdate) {
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        if (c < kk) {
-                            if (valid) lam[base + static_cast<size_t>(t0 + c) * kTile] = L[c];
-                            if (local) ep_lam[(t0 + c) * kTile + lane] = L[c];
-                        }
-                    }
-                }
+                for (int j = 0; j < C; ++j)
+                    if (j < kk) push_labels<W>(x, c[j], L[j]);
             }
-            term = fmaf(-omega, negsum, E);
         }
-
-        if constexpr (MODE == kBwdUpdate) {
-            // SP(r, v) over the whole row, one segment at a time; keep the labels at segment starts
-            {
-                float f[W];
+        if (u > 0) {
 #pragma unroll
-                for (int v = 0; v < W; ++v) f[v] = v == 0 ? 0.f : finf();
-                for (int s = 0; s < nseg; ++s) {
-                    const int t0 = s * C;
-                    const int kk = (k - t0 < C) ? k - t0 : C;
-                    float L[C];
-                    int V[C];
-                    fetch(s, L, V, false);
-#pragma unroll
-                    for (int v = 0; v < W; ++v) cp[(s * W + v) * kTile] = f[v];
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        if (c < kk) {
-                            uint32_t cd[W];
-                            load_codes<W>(tpl + (t0 + c) * W, cd);
-                            float nf[W];
-#pragma unroll
-                            for (int v = 0; v < W; ++v) nf[v] = finf();
-#pragma unroll
-                            for (int v = 0; v < W; ++v) {
-                                push<W>(nf, cd[v] & 0xFFu, f[v]);
-                                push<W>(nf, cd[v] >> 8, f[v] + L[c]);
-                            }
-#pragma unroll
-                            for (int v = 0; v < W; ++v) f[v] = nf[v];
-                        }
-                    }
-                }
-            }
-            float b[W];
-#pragma unroll
-            for (int v = 0; v < W; ++v) b[v] = finf();
-            float negsum = 0.f;
-            float Ln[C];
-            int Vn[C];
-            fetch(nseg - 1, Ln, Vn, true);
-            for (int s = nseg - 1; s >= 0; --s) {
-                const int t0 = s * C;
-                const int kk = (k - t0 < C) ? k - t0 : C;
-                float L[C], Tt[C], Sg[C][W];
-                int V[C];
-#pragma unroll
-                for (int c = 0; c < C; ++c) { L[c] = Ln[c]; V[c] = Vn[c]; }
-                if (s > 0) fetch(s - 1, Ln, Vn, true);  // in flight while this segment is swept
-                terms(L, V, Tt);
-                if (local && valid) {
-#pragma unroll
-                    for (int c = 0; c < C; ++c)
-                        if (c < kk) ep_var[(t0 + c) * kTile + lane] = V[c];
-                }
-                // labels of the segment's layers, from its checkpoint
-                {
-                    float f[W];
-#pragma unroll
-                    for (int v = 0; v < W; ++v) f[v] = cp[(s * W + v) * kTile];
-#pragma unroll
-                    for (int c = 0; c < C; ++c) {
-                        if (c < kk) {
-                            uint32_t cd[W];
-                            load_codes<W>(tpl + (t0 + c) * W, cd);
-                            float nf[W];
-#pragma unroll
-                            for (int v = 0; v < W; ++v) { Sg[c][v] = f[v]; nf[v] = finf(); }
-#pragma unroll
-                            for (int v = 0; v < W; ++v) {
-                                push<W>(nf, cd[v] & 0xFFu, f[v]);
-                                push<W>(nf, cd[v] >> 8, f[v] + L[c]);
-                            }
-#pragma unroll
-                            for (int v = 0; v < W; ++v) f[v] = nf[v];
-                        }
-                    }
-                }
-#pragma unroll
-                for (int cc = C - 1; cc >= 0; --cc) {
-                    if (cc < kk) {
-                        uint32_t cd[W];
-                        load_codes<W>(tpl + (t0 + cc) * W, cd);
-                        float m0 = finf(), m1 = finf();
-#pragma unroll
-                        for (int v = 0; v < W; ++v) {
-                            const float fv = Sg[cc][v];
-                            m0 = fminf(m0, fv + pick<W>(b, cd[v] & 0xFFu));
-                            m1 = fminf(m1, fv + pick<W>(b, cd[v] >> 8));
-                        }
-                        const float lt = L[cc];
-                        m1 += lt;
-                        const float d = m1 - m0;
-                        const float lt_new = fmaf(-omega, d, lt) + Tt[cc];  // Eq. 5
-                        L[cc] = lt_new;
-                        negsum += fmaxf(-d, 0.f);
-                        float nb[W];
-#pragma unroll
-                        for (int v = 0; v < W; ++v)
-                            nb[v] = fminf(pick<W>(b, cd[v] & 0xFFu), pick<W>(b, cd[v] >> 8) + lt_new);
-#pragma unroll
-                        for (int v = 0; v < W; ++v) b[v] = nb[v];
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    if (c < kk) {
-                        if (valid) lam[base + static_cast<size_t>(t0 + c) * kTile] = L[c];
-                        if (local) ep_lam[(t0 + c) * kTile + lane] = L[c];
-                    }
-                }
-            }
-            term = fmaf(-omega, negsum, b[0]);
+            for (int j = 0; j < C; ++j) { L[j] = Ln[j]; c[j] = cn[j]; }
         }
-
+    }
+    float term = 0.f;
+    if constexpr (MODE == kEval) {
+        term = x[0];
+    } else {
         if constexpr (update) {
-            if (local) {
-                __syncwarp();
-                tile_local_sums(I, tile.pattern, ep_lam, ep_var, lane);
-                __syncwarp();
-            }
+            fetch_terms(seg_of(0), V, T);
+            if (nseg > 1) fetch_var(seg_of(1), V);
         }
-
-        if constexpr (MODE == kBwdUpdate || MODE == kEval) {  // the passes whose bound is reduced
-            float s = valid ? term : 0.f, comp = 0.f;
+        float* __restrict__ mm0 = I->mm0;
+        float* __restrict__ mm1 = I->mm1;
+        float negsum = 0.f;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const float o = __shfl_xor_sync(kFull, s, off);
-                const float oc = __shfl_xor_sync(kFull, comp, off);
-                const float sum = s + o;
-                const float bp = sum - s;
-                const float err = (s - (sum - bp)) + (o - bp);
-                s = sum;
-                comp = comp + oc + err;
+        for (int v = 0; v < W; ++v) x[v] = asc && v == 0 ? 0.f : finf();
+        for (int u = 0; u < nseg; ++u) {
+            const int s = seg_of(u);
+            const int kk = min(k - s * C, C);
+            if (u + 1 < nseg) {  // in flight while this segment is swept
+                fetch_lam(seg_of(u + 1), Ln);
+                load_segment_codes<W>(tpl, seg_of(u + 1) * C, cn);
+                if constexpr (update) {
+                    fetch_terms(seg_of(u + 1), V, Tn);
+                    if (u + 2 < nseg) fetch_var(seg_of(u + 2), V);
+                }
             }
-            if (lane == 0) I->tile_lb[__ldg(a.first + ii) + (g - __ldg(a.prefix + ii))] = make_float2(s, comp);
+            // opposite labels of the segment's layers, from its checkpoint: S[j] holds those of the layer after j
+            // (asc) or of layer j (else)
+            float S[C][W], y[W];
+#pragma unroll
+            for (int v = 0; v < W; ++v) y[v] = cp[(s * W + v) * kTile];
+            if constexpr (asc) {
+#pragma unroll
+                for (int j = C - 1; j >= 0; --j) {
+                    if (j < kk) {
+#pragma unroll
+                        for (int v = 0; v < W; ++v) S[j][v] = y[v];
+                        if (j > 0) pull_labels<W>(y, c[j], L[j]);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    if (j < kk) {
+#pragma unroll
+                        for (int v = 0; v < W; ++v) S[j][v] = y[v];
+                        if (j + 1 < C) push_labels<W>(y, c[j], L[j]);
+                    }
+                }
+            }
+            if constexpr (asc) {
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    if (j < kk) {
+                        float m0, m1;
+                        layer_marginals<W>(x, S[j], c[j], m0, m1);
+                        m1 += L[j];
+                        if constexpr (MODE == kFwdUpdate) {
+                            L[j] = fmaf(-omega, m1 - m0, L[j]) + T[j];  // Eq. 5
+                        } else if (valid) {
+                            const size_t p = base + static_cast<size_t>(s * C + j) * kTile;
+                            if (a.flags & kMMBoth) { mm0[p] = m0; mm1[p] = m1; }
+                            else mm0[p] = m1 - m0;
+                        }
+                        push_labels<W>(x, c[j], L[j]);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int j = C - 1; j >= 0; --j) {
+                    if (j < kk) {
+                        float m0, m1;
+                        layer_marginals<W>(S[j], x, c[j], m0, m1);
+                        m1 += L[j];
+                        const float d = m1 - m0;
+                        L[j] = fmaf(-omega, d, L[j]) + T[j];  // Eq. 5
+                        negsum += fmaxf(-d, 0.f);
+                        pull_labels<W>(x, c[j], L[j]);
+                    }
+                }
+            }
+            if constexpr (update) {
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    if (j < kk) {
+                        if (valid) lam[base + static_cast<size_t>(s * C + j) * kTile] = L[j];
+                        if (local) ep_lam[(s * C + j) * kTile + lane] = L[j];
+                    }
+                }
+            }
+            if (u + 1 < nseg) {
+#pragma unroll
+                for (int j = 0; j < C; ++j) { L[j] = Ln[j]; T[j] = Tn[j]; c[j] = cn[j]; }
+            }
         }
+        if constexpr (!asc) term = fmaf(-omega, negsum, x[0]);
+    }
+
+    if constexpr (update) {
+        if (local) {
+            __syncwarp();
+            tile_local_sums(I, tile.pattern, ep_lam, ep_var, lane);
+            __syncwarp();
+        }
+    }
+    if constexpr (MODE == kBwdUpdate || MODE == kEval) {  // the passes whose bound is reduced
+        const float2 p = tile_bound(valid ? term : 0.f);
+        if (lane == 0) I->tile_lb[ti] = p;
     }
 }
 
@@ -967,27 +843,31 @@ template <int W>
 cudaError_t launch_sweep_width(bool reg, int mode, int blocks, int threads, size_t smem, cudaStream_t s,
                                const SweepArgs& a, const L2Window& l2);
 
-#define FDOG_DEFINE_SWEEP_WIDTH(W, HAS_REG)                                                                    \
+namespace dev {
+template <int W, bool REG>
+inline auto sweep_fn(int mode) -> void (*)(SweepArgs) {
+    return mode == kFwdUpdate ? sweep_kernel<W, REG, kFwdUpdate>
+         : mode == kBwdUpdate ? sweep_kernel<W, REG, kBwdUpdate>
+         : mode == kMinMarg   ? sweep_kernel<W, REG, kMinMarg>
+                              : sweep_kernel<W, REG, kEval>;
+}
+template <int W>
+inline auto seg_fn(int mode) -> void (*)(SweepArgs) {
+    return mode == kFwdUpdate ? sweep_seg_kernel<W, kFwdUpdate>
+         : mode == kBwdUpdate ? sweep_seg_kernel<W, kBwdUpdate>
+         : mode == kMinMarg   ? sweep_seg_kernel<W, kMinMarg>
+                              : sweep_seg_kernel<W, kEval>;
+}
+}  // namespace dev
+
+// narrow widths have the register and the segmented kernels, wide ones the shared-memory kernel
+#define FDOG_DEFINE_SWEEP_WIDTH(W)                                                                             \
     template <>                                                                                                \
     cudaError_t launch_sweep_width<W>(bool reg, int mode, int blocks, int threads, size_t smem, cudaStream_t s, \
                                       const SweepArgs& a, const L2Window& l2) {                                \
-        void (*fn)(SweepArgs) = nullptr;                                                                       \
-        if (HAS_REG && reg) {                                                                                  \
-            fn = mode == kFwdUpdate ? dev::sweep_kernel<W, HAS_REG, kFwdUpdate>                                \
-               : mode == kBwdUpdate ? dev::sweep_kernel<W, HAS_REG, kBwdUpdate>                                \
-               : mode == kMinMarg   ? dev::sweep_kernel<W, HAS_REG, kMinMarg>                                  \
-                                    : dev::sweep_kernel<W, HAS_REG, kEval>;                                    \
-        } else if (HAS_REG) {                                                                                  \
-            fn = mode == kFwdUpdate ? dev::sweep_seg_kernel<W, kFwdUpdate>                                     \
-               : mode == kBwdUpdate ? dev::sweep_seg_kernel<W, kBwdUpdate>                                     \
-               : mode == kMinMarg   ? dev::sweep_seg_kernel<W, kMinMarg>                                       \
-                                    : dev::sweep_seg_kernel<W, kEval>;                                         \
-        } else {                                                                                               \
-            fn = mode == kFwdUpdate ? dev::sweep_kernel<W, false, kFwdUpdate>                                  \
-               : mode == kBwdUpdate ? dev::sweep_kernel<W, false, kBwdUpdate>                                  \
-               : mode == kMinMarg   ? dev::sweep_kernel<W, false, kMinMarg>                                    \
-                                    : dev::sweep_kernel<W, false, kEval>;                                      \
-        }                                                                                                      \
+        void (*fn)(SweepArgs);                                                                                 \
+        if constexpr (W <= kRegW) fn = reg ? dev::sweep_fn<W, true>(mode) : dev::seg_fn<W>(mode);              \
+        else fn = dev::sweep_fn<W, false>(mode);                                                               \
         if (smem > 48 * 1024) {                                                                                \
             cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,              \
                                                  static_cast<int>(smem));                                      \

@@ -2,5 +2,5 @@
 #include "sweep.cuh"
 
 namespace fdog {
-FDOG_DEFINE_SWEEP_WIDTH(2, true)
+FDOG_DEFINE_SWEEP_WIDTH(2)
 }  // namespace fdog

@@ -2,5 +2,5 @@
 #include "sweep.cuh"
 
 namespace fdog {
-FDOG_DEFINE_SWEEP_WIDTH(8, false)
+FDOG_DEFINE_SWEEP_WIDTH(8)
 }  // namespace fdog
