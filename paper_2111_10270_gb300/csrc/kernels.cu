@@ -30,9 +30,13 @@ namespace {
 using dev::FlatArgs;
 using dev::LbArgs;
 using dev::block_pair_reduce;
+using dev::CommitIn;
+using dev::commit_in;
 using dev::commit_iteration;
 using dev::find_inst;
+using dev::kLbFew;
 using dev::lb_chunk;
+using dev::lb_few;
 using dev::lb_total;
 using dev::neumaier;
 using dev::reduce_T_one;
@@ -40,32 +44,41 @@ using dev::reduce_T_wide_one;
 
 // One block per chunk of kLbChunk tiles (chunk g of the flat batch), then the
 // last block of the instance sums the chunk partials and stages the bound for
-// lb_commit_kernel, or with `commit` commits the iteration itself.  The
-// chunking depends only on the instance, so its bound is the same alone or in
-// a batch.
+// lb_commit_kernel, or with `commit` commits the iteration itself.  An
+// instance of a few chunks is left to its first block.  The chunking depends
+// only on the instance, so its bound is the same alone or in a batch.
 __device__ __forceinline__ void lb_reduce_block(const LbArgs& a, int g, bool commit) {
     __shared__ double ss[8], sc[8];
-    __shared__ float ssf[8], scf[8];
+    __shared__ float ssf[kLbFew][8], scf[kLbFew][8];
     __shared__ int last;
     const int ii = find_inst(a.prefix, a.n_inst, g);
     const InstDev* __restrict__ I = a.insts + ii;
     InstCtl* ctl = I->ctl;
     if (FDOG_INACTIVE(ctl)) return;
     const int c = g - __ldg(a.prefix + ii);
-    const double chunk = lb_chunk(I, c, ssf, scf);
-    if (threadIdx.x == 0) {
-        I->chunk_lb[c] = chunk;
+    const int n_chunks = I->n_chunks;
+    CommitIn in;
+    if (threadIdx.x == 0 && commit) in = commit_in(ctl);
+    double lb;
+    if (n_chunks <= kLbFew) {
+        if (c > 0) return;
+        lb = lb_few(I, n_chunks, ssf, scf, ss);
+    } else {
+        const double chunk = lb_chunk(I, c, ssf[0], scf[0]);
+        if (threadIdx.x == 0) {
+            I->chunk_lb[c] = chunk;
+            __threadfence();
+            last = atomicAdd(&ctl->ticket, 1) == n_chunks - 1;
+        }
+        __syncthreads();
+        if (!last) return;
         __threadfence();
-        last = atomicAdd(&ctl->ticket, 1) == I->n_chunks - 1;
+        lb = lb_total(I, ss, sc);
     }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    const double lb = lb_total(I, ss, sc);
     if (threadIdx.x == 0) {
-        ctl->ticket = 0;
+        if (n_chunks > kLbFew) ctl->ticket = 0;
         if (commit) {
-            commit_iteration(ctl, lb);
+            commit_iteration(ctl, lb, in);
         } else {
             ctl->lb_staged = lb;
             ctl->staged = 1;
@@ -86,9 +99,12 @@ __global__ void __launch_bounds__(256) lb_reduce_kernel(LbArgs a) {
 // the rest: a thread per listed variable with at most 8 copies.  The parts
 // read only the pass's output and write disjoint state.  END: a commit may
 // land while the deferred sums run, so they test the instance's activity as
-// the ascending step recorded it at the start of the iteration.
+// the ascending step recorded it at the start of the iteration.  Held at 32
+// registers, eight blocks to an SM: the gathers of the many variables need the
+// warps (at 40 registers, which the bound's few blocks would like, the
+// descending step of the 512x512 grid took 20.6 us instead of 18.5).
 template <bool END>
-__global__ void __launch_bounds__(256) deferred_sum_kernel(FlatArgs work, FlatArgs wide, LbArgs l, int chunks,
+__global__ void __launch_bounds__(256, 8) deferred_sum_kernel(FlatArgs work, FlatArgs wide, LbArgs l, int chunks,
                                                            int wide_blocks) {
     dev::pdl_trigger();
     dev::pdl_wait();
@@ -122,7 +138,7 @@ __global__ void lb_commit_kernel(const InstDev* insts, int n) {
     InstCtl* ctl = insts[i].ctl;
     if (!ctl->staged) return;
     ctl->staged = 0;
-    commit_iteration(ctl, ctl->lb_staged);
+    commit_iteration(ctl, ctl->lb_staged, commit_in(ctl));
 }
 
 // C_i = c_i, T_i = 0 (M-bar = 0)

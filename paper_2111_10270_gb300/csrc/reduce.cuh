@@ -146,17 +146,34 @@ __device__ __forceinline__ void block_pair_reduce(double* ss, double* sc, double
     }
 }
 
+// What committing an iteration reads of the control block.  Nothing writes it
+// between the start of the launch and the commit, so the thread that commits
+// loads it before it forms the bound.
+struct CommitIn {
+    int iter, since, stop, window, min_iters;
+    double tol, prev;  // prev: the bound `window` iterations back
+};
+
+__device__ __forceinline__ CommitIn commit_in(const InstCtl* ctl) {
+    CommitIn c;
+    c.iter = ctl->iter;
+    c.since = ctl->since_reset;
+    c.stop = ctl->stop_enabled;
+    c.window = ctl->window;
+    c.min_iters = ctl->min_iters;
+    c.tol = ctl->tol;
+    c.prev = c.iter >= c.window ? ctl->lb_ring[(c.iter - c.window) % kLbRing] : 0.0;
+    return c;
+}
+
 // bound of a finished iteration: ring, counter, stopping test (Alg. 1 text)
-__device__ __forceinline__ void commit_iteration(InstCtl* ctl, double lb) {
-    const int it = ctl->iter;
-    ctl->lb_ring[it % kLbRing] = lb;
+__device__ __forceinline__ void commit_iteration(InstCtl* ctl, double lb, const CommitIn& c) {
+    ctl->lb_ring[c.iter % kLbRing] = lb;
     ctl->lb_last = lb;
-    ctl->iter = it + 1;
-    const int since = ++ctl->since_reset;
-    if (ctl->stop_enabled && since >= ctl->min_iters && since > ctl->window) {
-        const double prev = ctl->lb_ring[(it - ctl->window) % kLbRing];
-        if (lb - prev <= ctl->tol * fmax(fabs(lb), 1.0)) ctl->done = 1;
-    }
+    ctl->iter = c.iter + 1;
+    ctl->since_reset = c.since + 1;
+    if (c.stop && c.since + 1 >= c.min_iters && c.since + 1 > c.window && lb - c.prev <= c.tol * fmax(fabs(lb), 1.0))
+        ctl->done = 1;
 }
 
 // Variables with more than 8 copies (one assignment variable of a matching
@@ -208,6 +225,65 @@ __device__ __forceinline__ double lb_total(const InstDev* __restrict__ I, double
     double S = s, Cc = cp;
     neumaier(S, Cc, I->const_lb);
     return S + Cc;
+}
+
+// The bound of an instance of at most kLbFew chunks, by one block: chunk by
+// chunk the operations of lb_chunk (the chunks' butterflies side by side, so
+// their latencies overlap), then those of lb_total.  Sums with the zeros of
+// absent chunks change nothing and are left out.  It has no ticket and no
+// fence: of the 8.4 us that the end of an iteration took on a matching of
+// 1,169 tiles (5 chunks), they, the FP64 butterflies over empty lanes and the
+// control block's loads behind them were 3.2.  Valid in thread 0.
+constexpr int kLbFew = 8;
+__device__ __forceinline__ double lb_few(const InstDev* __restrict__ I, int n_chunks, float (*ss)[8], float (*sc)[8],
+                                         double* sd) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2 p[kLbFew];
+#pragma unroll
+    for (int q = 0; q < kLbFew; ++q) {
+        const int t = q * kLbChunk + threadIdx.x;
+        p[q] = q < n_chunks && t < I->n_tiles ? I->tile_lb[t] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+        for (int q = 0; q < kLbFew; ++q) {
+            if (q >= n_chunks) break;
+            const float os = __shfl_xor_sync(0xffffffffu, p[q].x, off);
+            const float oc = __shfl_xor_sync(0xffffffffu, p[q].y, off);
+            pair_add_f(p[q].x, p[q].y, os, oc);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kLbFew; ++q)
+        if (lane == 0) {
+            ss[q][w] = p[q].x;
+            sc[q][w] = p[q].y;
+        }
+    __syncthreads();
+    if (w < n_chunks) {  // warp w: the eight warps' parts of chunk w
+        float s = lane < 8 ? ss[w][lane] : 0.f, c = lane < 8 ? sc[w][lane] : 0.f;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) {
+            const float os = __shfl_xor_sync(0xffffffffu, s, off);
+            const float oc = __shfl_xor_sync(0xffffffffu, c, off);
+            pair_add_f(s, c, os, oc);
+        }
+        if (lane == 0) sd[w] = static_cast<double>(s) + static_cast<double>(c);
+    }
+    __syncthreads();
+    double S = 0.0, C = 0.0;
+    if (w == 0) {
+        if (lane < n_chunks) neumaier(S, C, sd[lane]);
+        for (int off = 4; off > 0; off >>= 1) {
+            if (off >= n_chunks) continue;
+            const double os = __shfl_xor_sync(0xffffffffu, S, off);
+            const double oc = __shfl_xor_sync(0xffffffffu, C, off);
+            neumaier_pair(S, C, os, oc);
+        }
+        neumaier(S, C, I->const_lb);
+    }
+    return S + C;
 }
 
 }  // namespace dev

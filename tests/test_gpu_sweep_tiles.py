@@ -72,3 +72,33 @@ def test_tile_edges(P, oracle_mod, name, shared, count):
     assert rel_err(m0[perm], om0).max() <= MM_RTOL and rel_err(m1[perm], om1).max() <= MM_RTOL
     _, fea = inst.lower_bound()
     assert lb_close(fea, orc.lower_bounds()[1], scale=np.abs(orc.energies()).sum())
+
+
+CTL_BYTES = 624
+
+
+@pytest.mark.parametrize("tiles", [1, 255, 256, 257, 512, 2047, 2048, 2049, 2305])
+def test_bound_of_any_number_of_chunks(P, oracle_mod, tiles):
+    """The bound is reduced by one block up to eight chunks of 256 tiles and by a block per chunk beyond; an
+    instance gets the same bound alone and beside one of the other kind."""
+    g = rows_ilp(*PATTERNS["product"], 32 * tiles - 5, tiles, False)
+    orc = oracle_mod.Problem.from_ilp(g)
+    params = P.capi.default_params(tol=0.0, jit=-1, max_rounds=0)
+    inst = P.Instance.from_ilp(g, params).build(0)
+    for _ in range(3):
+        done, lb = inst.iterate(1)
+        assert done == 1 and lb_close(lb, orc.iterate(1)[0]), tiles
+    other = P.Instance.from_ilp(rows_ilp(*PATTERNS["product"], 32 * (300 if tiles > 2048 else 3000), 7, False),
+                                params).build(0)
+    inst.reset()
+    b = P.Batch([inst, other])
+    iters, _, _ = b.solve(3)
+    assert list(iters) == [3, 3]
+    b.close()
+    alone = P.Instance.from_ilp(g, params).build(0)
+    alone.iterate(3)
+    alone.primal_round()
+    # the running bounds of the three iterations: the first entries of the control block that ends a checkpoint
+    ring = [np.frombuffer(x.export_state()[-CTL_BYTES:], np.float64, count=3) for x in (inst, alone)]
+    assert np.array_equal(ring[0], ring[1]) and np.all(ring[0] != 0)
+    assert all(np.array_equal(x, y) for x, y in zip(inst.multipliers(), alone.multipliers()))
