@@ -192,18 +192,71 @@ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
     return z ^ (z >> 31);
 }
 
-struct RoundArgs {
-    FlatArgs f;
-};
+// Alg. 2 for one variable with its copies' signs counted and M_ij summed: agreement
+// test, rounded value and the perturbation of this round.
+__device__ __forceinline__ void round_decide(const InstDev* __restrict__ I, int i, int cnt, int npos, int nneg,
+                                             int nzero, float sum) {
+    if (!(npos == cnt || nneg == cnt)) atomicAdd(&I->ctl->n_disagree, 1);
+    I->x[i] = sum < 0.f ? 1 : 0;
+    const int round = I->ctl->round;
+    const double delta = I->ctl->delta;
+    const uint64_t h = mix64(static_cast<uint64_t>(I->seed) ^
+                             (static_cast<uint64_t>(static_cast<uint32_t>(round)) << 32) ^
+                             static_cast<uint64_t>(static_cast<uint32_t>(i)));
+    // r uniform in [-delta, delta) (Alg. 2); the tie and conflict pushes are r * delta
+    const double r = (2.0 * (static_cast<double>(h >> 11) * 0x1.0p-53) - 1.0) * delta;
+    double p;
+    if (npos == cnt) p = delta;
+    else if (nneg == cnt) p = -delta;
+    else if (nzero == cnt) p = r * delta;
+    else {
+        const double sg = sum > 0.f ? 1.0 : (sum < 0.f ? -1.0 : (r >= 0.0 ? 1.0 : -1.0));
+        p = sg * fabs(r) * delta;
+    }
+    I->pert[i] = static_cast<float>(p);
+}
+
+// Variables with more copies than the deferred-sum buckets hold take a warp
+// each, as in the deferred sums (blocks [0, wide_blocks) of the two kernels
+// below); a thread walking the hundreds of copies of a matching's assignment
+// variable took 34 us to perturb and 12 us to test.
+__device__ __forceinline__ int wide_var(const FlatArgs& wide, const InstDev* __restrict__& I) {
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (g >= wide.total) return -1;
+    const int ii = find_inst(wide.prefix, wide.n_inst, g);
+    I = wide.insts + ii;
+    return I->work[I->wb_start[FDOG_WBUCKETS - 1] + (g - __ldg(wide.prefix + ii))];
+}
 
 // Alg. 2 per variable: agreement test on M_ij and the perturbation of this round
-__global__ void __launch_bounds__(256) round_test_kernel(RoundArgs a) {
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.f.total; g += gridDim.x * blockDim.x) {
-        const int ii = find_inst(a.f.prefix, a.f.n_inst, g);
-        const InstDev* __restrict__ I = a.f.insts + ii;
-        const int i = g - __ldg(a.f.prefix + ii);
+__global__ void __launch_bounds__(256) round_test_kernel(FlatArgs a, FlatArgs wide, int wide_blocks) {
+    if (static_cast<int>(blockIdx.x) < wide_blocks) {
+        const InstDev* __restrict__ I;
+        const int i = wide_var(wide, I);
+        if (i < 0) return;
+        const int lane = threadIdx.x & 31;
         const int b = I->csr_off[i], e = I->csr_off[i + 1];
-        if (b == e) continue;
+        int npos = 0, nneg = 0, nzero = 0;
+        float sum = 0.f;
+        for (int p0 = b; p0 < e; p0 += 32) {
+            const int n = min(32, e - p0);
+            const float m = lane < n ? I->mm0[I->csr_pos[p0 + lane]] : 0.f;
+            npos += __popc(__ballot_sync(0xffffffffu, lane < n && m > 0.f));
+            nneg += __popc(__ballot_sync(0xffffffffu, lane < n && m < 0.f));
+            nzero += __popc(__ballot_sync(0xffffffffu, lane < n && m == 0.f));
+            // one copy after the other, in ascending slot order as for every variable
+            for (int q = 0; q < n; ++q) sum += __shfl_sync(0xffffffffu, m, q);
+        }
+        if (lane == 0) round_decide(I, i, e - b, npos, nneg, nzero, sum);
+        return;
+    }
+    const int blocks = gridDim.x - wide_blocks;
+    for (int g = (blockIdx.x - wide_blocks) * blockDim.x + threadIdx.x; g < a.total; g += blocks * blockDim.x) {
+        const int ii = find_inst(a.prefix, a.n_inst, g);
+        const InstDev* __restrict__ I = a.insts + ii;
+        const int i = g - __ldg(a.prefix + ii);
+        const int b = I->csr_off[i], e = I->csr_off[i + 1];
+        if (b == e || e - b >= FDOG_WBUCKETS) continue;
         int npos = 0, nneg = 0, nzero = 0;
         float sum = 0.f;
         for (int p = b; p < e; ++p) {
@@ -213,37 +266,34 @@ __global__ void __launch_bounds__(256) round_test_kernel(RoundArgs a) {
             nzero += m == 0.f;
             sum += m;
         }
-        const int cnt = e - b;
-        if (!(npos == cnt || nneg == cnt)) atomicAdd(&I->ctl->n_disagree, 1);
-        I->x[i] = sum < 0.f ? 1 : 0;
-        const int round = I->ctl->round;
-        const double delta = I->ctl->delta;
-        const uint64_t h = mix64(static_cast<uint64_t>(I->seed) ^
-                                 (static_cast<uint64_t>(static_cast<uint32_t>(round)) << 32) ^
-                                 static_cast<uint64_t>(static_cast<uint32_t>(i)));
-        // r uniform in [-delta, delta) (Alg. 2); the tie and conflict pushes are r * delta
-        const double r = (2.0 * (static_cast<double>(h >> 11) * 0x1.0p-53) - 1.0) * delta;
-        double p;
-        if (npos == cnt) p = delta;
-        else if (nneg == cnt) p = -delta;
-        else if (nzero == cnt) p = r * delta;
-        else {
-            const double sg = sum > 0.f ? 1.0 : (sum < 0.f ? -1.0 : (r >= 0.0 ? 1.0 : -1.0));
-            p = sg * fabs(r) * delta;
-        }
-        I->pert[i] = static_cast<float>(p);
+        round_decide(I, i, e - b, npos, nneg, nzero, sum);
     }
 }
 
 // Alg. 2: lambda^j_i += p_i for all j in J_i (only if some variable disagrees)
-__global__ void __launch_bounds__(256) round_apply_kernel(FlatArgs a) {
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.total; g += gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(256) round_apply_kernel(FlatArgs a, FlatArgs wide, int wide_blocks) {
+    if (static_cast<int>(blockIdx.x) < wide_blocks) {
+        const InstDev* __restrict__ I;
+        const int i = wide_var(wide, I);
+        if (i < 0 || I->ctl->n_disagree == 0) return;
+        const int lane = threadIdx.x & 31;
+        const int b = I->csr_off[i], e = I->csr_off[i + 1];
+        const float p = I->pert[i];
+        for (int q = b + lane; q < e; q += 32) I->lam[I->csr_pos[q]] += p;
+        if (lane == 0) {
+            I->C[i] += p * static_cast<float>(e - b);
+            I->T[i] = 0.f;
+        }
+        return;
+    }
+    const int blocks = gridDim.x - wide_blocks;
+    for (int g = (blockIdx.x - wide_blocks) * blockDim.x + threadIdx.x; g < a.total; g += blocks * blockDim.x) {
         const int ii = find_inst(a.prefix, a.n_inst, g);
         const InstDev* __restrict__ I = a.insts + ii;
         if (I->ctl->n_disagree == 0) continue;
         const int i = g - __ldg(a.prefix + ii);
         const int b = I->csr_off[i], e = I->csr_off[i + 1];
-        if (b == e) continue;
+        if (b == e || e - b >= FDOG_WBUCKETS) continue;
         const float p = I->pert[i];
         for (int q = b; q < e; ++q) I->lam[I->csr_pos[q]] += p;
         I->C[i] += p * static_cast<float>(e - b);
@@ -670,16 +720,18 @@ cudaError_t launch_zero_T(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t 
 cudaError_t launch_round_test(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s) {
     if (b.vars_total == 0) return cudaSuccess;
     cfg.count();
-    round_test_kernel<<<blocks_for(b.vars_total, 256, cfg.num_sms * 8), 256, 0, s>>>(
-        RoundArgs{flat(b, b.var_prefix, b.vars_total)});
+    const int wide_blocks = (b.wide_total + 7) / 8;  // 8 warps per block
+    round_test_kernel<<<wide_blocks + blocks_for(b.vars_total, 256, cfg.num_sms * 8), 256, 0, s>>>(
+        flat(b, b.var_prefix, b.vars_total), flat(b, b.wide_prefix, b.wide_total), wide_blocks);
     return cudaGetLastError();
 }
 
 cudaError_t launch_round_apply(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s) {
     if (b.vars_total == 0) return cudaSuccess;
     cfg.count();
-    round_apply_kernel<<<blocks_for(b.vars_total, 256, cfg.num_sms * 8), 256, 0, s>>>(
-        flat(b, b.var_prefix, b.vars_total));
+    const int wide_blocks = (b.wide_total + 7) / 8;
+    round_apply_kernel<<<wide_blocks + blocks_for(b.vars_total, 256, cfg.num_sms * 8), 256, 0, s>>>(
+        flat(b, b.var_prefix, b.vars_total), flat(b, b.wide_prefix, b.wide_total), wide_blocks);
     return cudaGetLastError();
 }
 
