@@ -103,3 +103,41 @@ def test_noalloc_bound_reduce_rejects_bad_arguments(env):
     assert L.fdog_bound_reduce_noalloc(p, -1, 0.0, p, s) == P.FDOG_EINVAL
     assert L.fdog_bound_reduce_noalloc(ctypes.c_void_p(0), 5, 0.0, p, s) == P.FDOG_EINVAL
     assert L.fdog_bound_reduce_noalloc(p, 1, 0.0, ctypes.c_void_p(0), s) == P.FDOG_EINVAL
+
+
+@pytest.mark.parametrize("n", [1, 3, 1024, 1025, (1 << 20) - 1, 1 << 20, (1 << 20) + 1, 4096 * 300 + 17])
+@pytest.mark.parametrize("kind", ["spread", "cancel", "tiny", "negative", "one"])
+def test_noalloc_bound_reduce_values(env, n, kind):
+    """Values of very different exponents, sums that cancel, subnormal values and a lone value among zeros, at the
+    sizes where the values per thread change: the fixed-point sum drops only what is 2^-112 of the largest value and
+    rounds once at the end, so it is within an ulp of the result and n 2^-110 of the largest value."""
+    torch = env[0]
+    rng = np.random.default_rng(n)
+    v = rng.standard_normal(n)
+    if kind == "spread":
+        v *= 2.0 ** rng.integers(-300, 301, n)
+    elif kind == "cancel":
+        v = np.where(np.arange(n) % 2 == 0, v, -np.roll(v, 1)) * 1e150
+    elif kind == "tiny":
+        v *= 5e-324 * rng.integers(1, 1000, n)
+    elif kind == "negative":
+        v = -np.abs(v)
+    else:
+        v = np.zeros(n)
+        v[n // 2] = -3.25e-200
+    dev = torch.from_numpy(v).to("cuda:0")
+    for constant in (0.0, -1.5):
+        got = reduce_noalloc(env, dev, n, constant)
+        want = math.fsum(list(v) + [constant])
+        bound = 2.0 ** -52 * abs(want) + n * 2.0 ** -110 * float(np.abs(v).max()) + 5e-324
+        assert abs(got - want) <= bound, (got, want, bound)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan")])
+def test_noalloc_bound_reduce_not_finite(env, bad):
+    torch = env[0]
+    v = torch.ones(5000, dtype=torch.float64, device="cuda:0")
+    v[4999] = bad
+    assert math.isnan(reduce_noalloc(env, v, 5000, 1.0))
+    v[4999] = 1.0
+    assert reduce_noalloc(env, v, 5000, 1.0) == 5001.0
