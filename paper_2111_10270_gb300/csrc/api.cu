@@ -213,7 +213,8 @@ static int plan_for_build(fdog_instance* inst) {
 int ensure_host_plan(fdog_instance* inst) {
     Decomposition& d = inst->dec;
     if (!d.on_device) return FDOG_OK;
-    if (!inst->arena || !d.d_bdd_row) return FDOG_ESTATE;
+    const int32_t* rows = d.d_bdd_row ? d.d_bdd_row : inst->slot_row;  // (slots.cu)
+    if (!inst->arena || !rows) return FDOG_ESTATE;
     DeviceGuard g(inst->device);
     const int64_t n = inst->n_vars;
     try {
@@ -238,7 +239,7 @@ int ensure_host_plan(fdog_instance* inst) {
     down(d.work.data(), a.work, sizeof(int32_t) * d.work.size());
     down(d.wpos.data(), a.wpos, sizeof(int32_t) * d.wpos.size());
     down(d.local_ent.data(), a.local_ent, sizeof(uint16_t) * d.local_ent.size());
-    down(d.bdd_row.data(), d.d_bdd_row, sizeof(int32_t) * d.bdd_row.size());
+    down(d.bdd_row.data(), rows, sizeof(int32_t) * d.bdd_row.size());
     if (e == cudaSuccess) e = cudaStreamSynchronize(inst->stream);
     if (e != cudaSuccess) return fail_cuda(inst, e, "plan download");
     d.bdd_shape.resize(d.n_bdds);
@@ -460,6 +461,7 @@ int release_device(fdog_instance* inst) {
     inst->engine = nullptr;
     if (inst->arena) cudaFree(inst->arena);
     if (inst->dev.mm1) cudaFree(inst->dev.mm1);
+    free_slots(inst);
     if (inst->host_ctl) cudaFreeHost(inst->host_ctl);
     if (inst->solution_pinned && inst->host_x) {
         inst->solution.assign(inst->host_x, inst->host_x + inst->n_vars);  // keep the last solution
@@ -972,46 +974,13 @@ int fdog_lower_bound(fdog_instance* inst, double* lb_running, double* lb_feasibl
     return FDOG_OK;
 }
 
-static int slot_table(fdog_instance* inst, int64_t* n_slots, int32_t* var, int32_t* row) {
-    const Decomposition& d = inst->dec;
-    if (!var) { *n_slots = d.n_slots; return FDOG_OK; }
-    if (*n_slots < d.n_slots) return FDOG_EINVAL;
-    int rc = ensure_host_plan(inst);
-    if (rc != FDOG_OK) return rc;
-    int64_t q = 0;
-    for (const TileDev& t : d.tiles) {
-        const int k = d.shapes[t.shape].k;
-        for (int l = 0; l < t.n_valid; ++l)
-            for (int layer = 0; layer < k; ++layer) {
-                const int64_t p = t.slot_base + static_cast<int64_t>(layer) * kTile + l;
-                var[q] = d.var[p];
-                if (row) row[q] = d.bdd_row[t.bdd_base + l];
-                ++q;
-            }
-    }
-    *n_slots = q;
-    return FDOG_OK;
-}
-
-static int gather_slots(fdog_instance* inst, const float* dev, float* out) {
-    const Decomposition& d = inst->dec;
-    std::vector<float> h(d.slots_pad);
-    cudaError_t e = copy_async(inst, h.data(), dev, sizeof(float) * d.slots_pad, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(inst->stream);
-    if (e != cudaSuccess) return fail_cuda(inst, e, "copy slots");
-    int64_t q = 0;
-    for (const TileDev& t : d.tiles) {
-        const int k = d.shapes[t.shape].k;
-        for (int l = 0; l < t.n_valid; ++l)
-            for (int layer = 0; layer < k; ++layer) out[q++] = h[t.slot_base + static_cast<int64_t>(layer) * kTile + l];
-    }
-    return FDOG_OK;
-}
-
 int fdog_min_marginals(fdog_instance* inst, int64_t* n_slots, int32_t* var, int32_t* row, float* m0, float* m1) {
     if (!inst || !n_slots) return FDOG_EINVAL;
     if (!inst->built) return FDOG_ESTATE;
-    if (!var) return slot_table(inst, n_slots, nullptr, nullptr);
+    if (!var) {
+        *n_slots = inst->dec.n_slots;
+        return FDOG_OK;
+    }
     if (*n_slots < inst->dec.n_slots) return FDOG_EINVAL;
     DeviceGuard g(inst->device);
     int rc = ensure_mm1(inst);
@@ -1020,20 +989,22 @@ int fdog_min_marginals(fdog_instance* inst, int64_t* n_slots, int32_t* var, int3
         cudaError_t e = launch_sweep(inst->batch, kMinMarg, kMMBoth, inst->cfg, inst->stream);
         if (e != cudaSuccess) return fail_cuda(inst, e, "min-marginals");
     }
-    if ((rc = slot_table(inst, n_slots, var, row)) != FDOG_OK) return rc;
-    if (m0 && (rc = gather_slots(inst, inst->dev.mm0, m0)) != FDOG_OK) return rc;
-    if (m1 && (rc = gather_slots(inst, inst->dev.mm1, m1)) != FDOG_OK) return rc;
-    return FDOG_OK;
+    rc = read_slots(inst, var, row, inst->dev.mm0, m0, inst->dev.mm1, m1);
+    if (rc == FDOG_OK) *n_slots = inst->dec.n_slots;
+    return rc;
 }
 
 int fdog_multipliers(fdog_instance* inst, int64_t* n_slots, int32_t* var, int32_t* row, float* lambda) {
     if (!inst || !n_slots) return FDOG_EINVAL;
     if (!inst->built) return FDOG_ESTATE;
-    if (!var) return slot_table(inst, n_slots, nullptr, nullptr);
+    if (!var) {
+        *n_slots = inst->dec.n_slots;
+        return FDOG_OK;
+    }
     if (*n_slots < inst->dec.n_slots) return FDOG_EINVAL;
     DeviceGuard g(inst->device);
-    int rc = slot_table(inst, n_slots, var, row);
-    if (rc == FDOG_OK && lambda) rc = gather_slots(inst, inst->dev.lam, lambda);
+    const int rc = read_slots(inst, var, row, inst->dev.lam, lambda, nullptr, nullptr);
+    if (rc == FDOG_OK) *n_slots = inst->dec.n_slots;
     return rc;
 }
 
@@ -1083,7 +1054,8 @@ int fdog_info(fdog_instance* inst, int64_t* n_vars, int64_t* n_bdds, int64_t* n_
     if (n_nodes) *n_nodes = inst->dec.n_nodes;
     if (device_bytes)
         *device_bytes = static_cast<int64_t>(inst->built ? inst->arena_bytes : arena_size(inst)) +
-                        (inst->dev.mm1 ? static_cast<int64_t>(sizeof(float) * inst->dec.slots_pad) : 0);
+                        (inst->dev.mm1 ? static_cast<int64_t>(sizeof(float) * inst->dec.slots_pad) : 0) +
+                        static_cast<int64_t>(inst->slot_bytes);
     return FDOG_OK;
 }
 
@@ -1106,6 +1078,7 @@ void fdog_destroy(fdog_instance* inst) {
         }
         if (inst->arena) cudaFree(inst->arena);
         if (inst->dev.mm1) cudaFree(inst->dev.mm1);
+        free_slots(inst);
         if (inst->host_ctl) cudaFreeHost(inst->host_ctl);
         if (inst->host_x) cudaFreeHost(inst->host_x);
         delete inst->self_view;

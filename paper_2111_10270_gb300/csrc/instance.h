@@ -85,6 +85,12 @@ struct fdog_instance {
     fdog::InstDev hdesc{};
     fdog::DevBatch batch;
     fdog::LaunchCfg cfg;
+    // slots in the order the C ABI lists them, made when first read (slots.cu): per tile its first slot in that
+    // order, per BDD its row, and one array of slots to gather into
+    int32_t* slot_first = nullptr;
+    int32_t* slot_row = nullptr;
+    int32_t* slot_out = nullptr;
+    size_t slot_bytes = 0;
     fdog::InstCtl* host_ctl = nullptr;  // pinned
     uint8_t* host_x = nullptr;          // pinned staging of the rounded solution
     bool solution_pinned = false;       // the last solution lives in host_x (else in `solution`)
@@ -139,4 +145,9 @@ int addback(fdog_instance* inst);
 // against the plan, and the initial multipliers of the shared variables
 int shard_check_copies(fdog_instance* inst);
 cudaError_t launch_shard_init(fdog_instance* inst);
+// the instance's slots (slots.cu): arrays of n_slots entries to the caller's host memory (any may be null);
+// on return they are complete.  free_slots releases what the first read made.
+int read_slots(fdog_instance* inst, int32_t* var, int32_t* row, const float* dev0, float* out0, const float* dev1,
+               float* out1);
+void free_slots(fdog_instance* inst);
 }  // namespace fdog

@@ -102,3 +102,38 @@ def test_bound_of_any_number_of_chunks(P, oracle_mod, tiles):
     ring = [np.frombuffer(x.export_state()[-CTL_BYTES:], np.float64, count=3) for x in (inst, alone)]
     assert np.array_equal(ring[0], ring[1]) and np.all(ring[0] != 0)
     assert all(np.array_equal(x, y) for x, y in zip(inst.multipliers(), alone.multipliers()))
+
+
+@pytest.mark.parametrize("planner", [0, 1], ids=["device plan", "host plan"])
+@pytest.mark.parametrize("count", [1, 33, 10921, 10923])
+def test_slots_as_listed(P, planner, count):
+    """Slots come tile by tile, BDD by BDD and layer by layer, below and above the number (65,536) from which each
+    array is copied by itself: six-variable rows in their order after four-variable ones (two shapes)."""
+    g = rows_ilp(*PATTERNS["card6"], count, 3, False)
+    few = rows_ilp(*PATTERNS["amo2"], 3, 4, False)
+    g.cost = np.concatenate([few.cost, g.cost])
+    g.row_ptr = np.concatenate([few.row_ptr, g.row_ptr[1:] + len(few.col)])
+    g.col = np.concatenate([few.col, g.col + few.n_vars]).astype(np.int32)
+    g.coef, g.sense, g.rhs = (np.concatenate([a, b]) for a, b in
+                              ((few.coef, g.coef), (few.sense, g.sense), (few.rhs, g.rhs)))
+    g.n_vars += few.n_vars
+    inst = P.Instance.from_ilp(g, P.capi.default_params(tol=0.0, jit=-1, planner=planner)).build(0)
+    inst.iterate(2)
+    for again in range(2):
+        var, row, m0, m1 = inst.min_marginals()
+        assert np.array_equal(var, g.col) and np.array_equal(row, np.repeat(np.arange(g.n_rows), np.diff(g.row_ptr)))
+        v2, r2, lam = inst.multipliers()
+        assert np.array_equal(v2, var) and np.array_equal(r2, row)
+        # rows share no variable: after two iterations a slot's multiplier is its variable's cost again plus what is
+        # pending, and the min-marginals of the rows are those of the listed multipliers
+        k = 6
+        x = lam[len(few.col):].reshape(count, k).astype(np.float64)
+        best = np.sort(x, 1)
+        base = np.minimum(np.cumsum(best, 1)[:, :3], 0).min(1)
+        got = np.minimum(m0, m1)[len(few.col):].reshape(count, k)
+        assert np.allclose(got, base[:, None], rtol=1e-5, atol=1e-5)
+        if again == 0:
+            inst.row_bdd(0)  # brings a device-built plan to the host
+            blob = inst.export_state()
+            inst.release()
+            inst.build(0).import_state(blob)
