@@ -61,6 +61,7 @@ static std::vector<Item> arena_items(const fdog_instance* inst, DevArrays& a) {
     const int64_t nchunks = std::max<int64_t>(1, (nt + kLbChunk - 1) / kLbChunk);
     const int64_t nobj = std::max<int64_t>(1, (n + kObjChunk - 1) / kObjChunk);
     auto sz = [](int64_t v) { return static_cast<size_t>(std::max<int64_t>(v, 1)); };
+    const bool bulk = bulk_wanted(inst) && !d.bulk_runs.empty();
     return {
         {reinterpret_cast<void**>(&a.inst), sizeof(InstDev)},
         {reinterpret_cast<void**>(&a.ctl), sizeof(InstCtl)},
@@ -79,6 +80,9 @@ static std::vector<Item> arena_items(const fdog_instance* inst, DevArrays& a) {
         {reinterpret_cast<void**>(&a.csr_pos), sizeof(int32_t) * sz(d.n_slots)},
         {reinterpret_cast<void**>(&a.patterns), sizeof(int32_t) * std::max<size_t>(d.patterns.size(), 2)},
         {reinterpret_cast<void**>(&a.local_ent), sizeof(uint16_t) * static_cast<size_t>(std::max<int64_t>(d.n_local_ent, 4))},
+        {reinterpret_cast<void**>(&a.cv), bulk ? sizeof(float) * kTile * static_cast<size_t>(d.bulk_cv_rows) : 0},
+        {reinterpret_cast<void**>(&a.bulk_pairs), bulk ? sizeof(uint32_t) * d.bulk_pairs.size() : 0},
+        {reinterpret_cast<void**>(&a.bulk_runs), bulk ? sizeof(BulkRun) * d.bulk_runs.size() : 0},
         {reinterpret_cast<void**>(&a.work), sizeof(int32_t) * sz(d.n_work)},
         {reinterpret_cast<void**>(&a.wpos), sizeof(int32_t) * sz(d.n_wpos)},
         {reinterpret_cast<void**>(&a.lab), sizeof(float) * static_cast<size_t>(std::max<int64_t>(d.lab_floats, 1))},
@@ -161,6 +165,7 @@ int plan(fdog_instance* inst, bool compile_jit) {
     inst->planned_on_device = false;
     if ((rc = check_layer_limits(inst)) != FDOG_OK) return rc;
     if (inst->params.update == 1) build_serial_schedule(inst->n_vars, inst->dec);
+    if (bulk_wanted(inst) && bulk_possible(inst->dec)) plan_bulk(inst->dec, inst->dec.local_ent.data());
     std::vector<int> ids = jit_ids(inst);
     if (compile_jit && !ids.empty()) {
         std::string why;
@@ -298,6 +303,13 @@ int allocate_and_upload(fdog_instance* inst) {
     h.csr_pos = a.csr_pos;
     h.patterns = a.patterns;
     h.local_ent = a.local_ent;
+    if (bulk_wanted(inst) && !d.bulk_runs.empty()) {
+        h.cv = a.cv;
+        h.bulk_runs = a.bulk_runs;
+        h.n_bulk_runs = static_cast<int32_t>(d.bulk_runs.size());
+        h.bulk_first = d.cls_tile_begin[kJitClass];
+        h.bulk_tiles = d.cls_tile_begin[kJitClass + 1] - d.cls_tile_begin[kJitClass];
+    }
     h.work = a.work;
     h.wpos = a.wpos;
     h.lab = a.lab;
@@ -361,6 +373,7 @@ int allocate_and_upload(fdog_instance* inst) {
     two(&b.wide_prefix, d.wb_start[FDOG_WBUCKETS] - d.wb_start[FDOG_WBUCKETS - 1]);
     b.wide_total = d.wb_start[FDOG_WBUCKETS] - d.wb_start[FDOG_WBUCKETS - 1];
     for (int c = 0; c < kNumClasses; ++c) b.has_local[c] = d.cls_has_local[c];
+    b.any_cv = h.cv != nullptr;
     two(&b.slot_prefix, static_cast<int32_t>(S));
     b.slots_total = static_cast<int32_t>(S);
     two(&b.chunk_prefix, static_cast<int32_t>(nt > 0 ? nchunks : 0));
@@ -421,7 +434,7 @@ int allocate_and_upload(fdog_instance* inst) {
         up(a.sh_slot, slot.data(), sizeof(int32_t) * slot.size());
     }
     if (e != cudaSuccess) return fail_cuda(inst, e, "upload");
-    return FDOG_OK;
+    return setup_bulk(inst);
 }
 
 // The engine and one-member view behind an instance's own calls.
@@ -478,6 +491,7 @@ int release_device(fdog_instance* inst) {
     inst->built = false;
     inst->pending_T = false;
     inst->iterated = false;
+    inst->terms_stale = false;
     return FDOG_OK;
 }
 
@@ -490,11 +504,13 @@ int reset_dual_state(fdog_instance* inst) {
     c.tol = p.tol;
     c.iter_limit = inst->shard ? INT32_MAX : 0;  // a shard's passes are driven by fdog_shard_pass
     c.delta = p.delta;
+    c.t_zero = 1;
     cudaError_t e = copy_async(inst, inst->dev.ctl, &c, sizeof(c), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return fail_cuda(inst, e, "reset ctl");
     e = launch_init(inst->batch, inst->cfg, inst->stream);
     if (e == cudaSuccess && inst->shard) e = launch_shard_init(inst);
     if (e != cudaSuccess) return fail_cuda(inst, e, "init");
+    inst->terms_stale = false;
     inst->pending_T = false;
     inst->iterated = false;
     return FDOG_OK;
@@ -522,7 +538,8 @@ int set_ctl_field(fdog_instance* inst, size_t offset, const void* v, size_t byte
 // Energy sum (+ presolve constant) at lambda, or at lambda + T (the add-back),
 // with FP64 shortest-path labels and FP64 compensated sums (eval.cu).
 int evaluate(fdog_instance* inst, bool add_t, double* out) {
-    cudaError_t e = launch_eval64(inst->batch, add_t, inst->cfg, inst->stream);
+    cudaError_t e = add_t ? flush_terms({inst}, inst->batch, inst->cfg, inst->stream) : cudaSuccess;
+    if (e == cudaSuccess) e = launch_eval64(inst->batch, add_t, inst->cfg, inst->stream);
     if (e != cudaSuccess) return fail_cuda(inst, e, "evaluate");
     InstCtl c;
     int rc = read_ctl(inst, c);
@@ -533,7 +550,8 @@ int evaluate(fdog_instance* inst, bool add_t, double* out) {
 
 int addback(fdog_instance* inst) {
     if (!inst->pending_T) return FDOG_OK;
-    cudaError_t e = launch_addback(inst->batch, inst->cfg, inst->stream);
+    cudaError_t e = flush_terms({inst}, inst->batch, inst->cfg, inst->stream);
+    if (e == cudaSuccess) e = launch_addback(inst->batch, inst->cfg, inst->stream);
     if (e != cudaSuccess) return fail_cuda(inst, e, "add-back");
     inst->pending_T = false;
     inst->iterated = false;

@@ -85,7 +85,11 @@ int view_build(Engine& e, BatchView& v, const std::vector<fdog_instance*>& membe
             if (s.jit >= 0) ids.push_back(s.jit);
     }
     b.insts = reinterpret_cast<InstDev*>(dbase);
-    if (n == 1) b.l2 = members[0]->batch.l2;  // the instance's deferred terms stay in L2 during its sweeps
+    if (n == 1) {
+        b.l2 = members[0]->batch.l2;  // the instance's deferred terms stay in L2 during its sweeps
+        b.bulk = members[0]->batch.bulk;
+    }
+    for (const fdog_instance* m : members) b.any_cv = b.any_cv || m->hdesc.cv;
     for (int c = 0; c < kNumClasses; ++c) {
         int32_t* pre = ints + q;
         int32_t* first = ints + q + n + 1;
@@ -157,6 +161,17 @@ int view_build(Engine& e, BatchView& v, const std::vector<fdog_instance*>& membe
     return FDOG_OK;
 }
 
+cudaError_t flush_terms(const std::vector<fdog_instance*>& members, const DevBatch& b, const LaunchCfg& cfg,
+                        cudaStream_t s) {
+    bool stale = false;
+    for (fdog_instance* m : members) stale = stale || m->terms_stale;
+    if (!stale) return cudaSuccess;
+    const cudaError_t e = launch_local_terms(b, cfg, s);
+    if (e == cudaSuccess)
+        for (fdog_instance* m : members) m->terms_stale = false;
+    return e;
+}
+
 int view_status(Engine& e, BatchView& v, std::vector<InstStatus>& out) {
     const int n = v.b.n_inst;
     out.resize(n);
@@ -205,6 +220,13 @@ int view_op(Engine& e, BatchView& v, int op, int arg) {
 
 int view_iterate(Engine& e, BatchView& v, int k) {
     if (k <= 0 || v.b.n_inst == 0) return FDOG_OK;
+    const bool bulk = v.b.bulk.ready;
+    if (!bulk && flush_terms(v.members, v.b, e.cfg, e.stream) != cudaSuccess) {
+        e.err = "pending terms";
+        cudaGetLastError();
+        return FDOG_ECUDA;
+    }
+    if (bulk) v.members[0]->terms_stale = true;
     if (e.persistent && !(e.prof && e.prof->on) && persist_supported(v.b)) {
         // the k iterations as one cooperative launch with grid barriers
         if (!e.dev_bar && cudaMalloc(reinterpret_cast<void**>(&e.dev_bar), 4 * sizeof(unsigned)) != cudaSuccess) {
@@ -276,7 +298,8 @@ int fail(Engine& e, cudaError_t ce, const char* where) {
 
 // add-back of Alg. 1 (lambda += T, T = 0) for every member
 int addback_all(Engine& e, BatchView& v) {
-    cudaError_t ce = launch_addback(v.b, e.cfg, e.stream);
+    cudaError_t ce = flush_terms(v.members, v.b, e.cfg, e.stream);
+    if (ce == cudaSuccess) ce = launch_addback(v.b, e.cfg, e.stream);
     if (ce != cudaSuccess) return fail(e, ce, "add-back");
     for (fdog_instance* m : v.members) {
         m->pending_T = false;
@@ -520,9 +543,14 @@ int view_autotune(Engine& e, BatchView& v, bool tune_grid) {
     };
     save(false);
     int rc = ce == cudaSuccess ? view_op(e, v, kOpLimit, 1 << 30) : FDOG_OK;
-    // warps per block x grid mode (one persistent wave, or a block per tile group)
+    // warps per block x grid mode (one persistent wave, or a block per tile group); bulk sweeps have a shape of their
+    // own, so a view with no other class is timed once, at the shape its other sweeps of such sizes like
+    int classes = 0;
+    for (int c = 0; c < kNumClasses; ++c) classes += v.b.tiles_total[c] > 0;
+    const bool fixed = tune_grid && v.b.bulk.ready && classes == 1;
     for (int combo = 0; combo < (tune_grid ? 6 : 3) && ce == cudaSuccess && rc == FDOG_OK; ++combo) {
         const int wpb = 2 << (combo % 3), waves = tune_grid ? (combo < 3 ? 1 : 0) : e.cfg.max_waves;
+        if (fixed && combo != 4) continue;  // 4 warps per block, a block per tile group
         cfg.warps_per_block = wpb;
         cfg.max_waves = waves;
         ce = launch_sweep(v.b, kFwdUpdate, 0, cfg, e.stream);  // warm-up

@@ -43,7 +43,6 @@ constexpr int kNumWidths = 4;
 constexpr int kMaxWidth = 16;
 constexpr int kMaxLayersSmem = 256;  // longest row the staged shared-memory kernels take
 constexpr int kMaxLayersSeg = 4096;  // longest row the segmented kernels (narrow BDDs) take
-constexpr int kEpiMaxK = 16;         // longest row whose tile can form tile-local deferred terms
 constexpr int kNumStaticClasses = 2 * kNumWidths;  // (width index) x (register | smem)
 constexpr int kJitClass = kNumStaticClasses;         // shape-specialised kernels
 constexpr int kNumClasses = kNumStaticClasses + 1;
@@ -79,6 +78,8 @@ struct TileDev {
     int32_t pad[3];
 };
 
+#define FDOG_EPI_LAYERS 16  // longest row whose tile can have tile-local variables
+
 #define FDOG_LB_RING 64
 #define FDOG_LB_CHUNK 256      // tiles per chunk of the lower-bound reduction
 
@@ -107,7 +108,8 @@ struct InstCtl {
     double lb_staged;
     int32_t pass_active;      // the instance's activity at the start of the running iteration, recorded
                               // by its ascending pass's deferred sums for the end-of-iteration kernel
-    int32_t pad;
+    int32_t t_zero;           // every deferred term is 0 (set up, added back or perturbed, no pass since): the
+                              // bulk sweeps then do not form those of tile-local variables from the multipliers
 };
 
 // True when the update kernels must leave the instance alone: its stopping
@@ -129,6 +131,11 @@ struct InstDev {
     float* mm1;              // [slots_pad] min-marginal output m1
     float* T;                // [n] deferred term  omega/|J_i| sum_k Mbar_ik
     float* C;                // [n] target sum_j lambda^j_i (= c_i, perturbed by rounding)
+    float* cv;               // bulk sweeps: per tile its targets and ids (see BulkRun), null without
+    const struct BulkRun* bulk_runs;
+    int32_t n_bulk_runs;
+    int32_t bulk_first;      // first tile of the class of those runs
+    int32_t bulk_tiles;      // and its tiles
     const int32_t* csr_off;  // [n + 1]
     const int32_t* csr_pos;  // [slots] padded slot positions of each variable, ascending
     const int32_t* patterns; // [2 per pattern] {first entry, entries}: variables whose copies all lie in one tile
@@ -177,8 +184,50 @@ struct SweepArgs {
                             // deferred sums (0: no tile of this launch has local variables)
 };
 
+// Bulk sweeps (jit_skeleton.cuh): the tiles of one shape of the
+// shape-specialised class lie one after the other, and so do their slots.
+// What a pass reads of a tile besides its multipliers lies in one block of
+// InstDev::cv: the targets C of the layers c_lo .. c_lo + c_n - 1, which hold
+// every tile-local slot of the run, then the ids of the layers v_lo .. v_lo +
+// v_n - 1, which hold every other slot (rows of 32, as the slots).
+#define FDOG_BULK_RUNS 16
+struct BulkRun {
+    int32_t tile;       // first tile, counted within the class
+    int32_t slot_base;  // its first slot
+    int32_t n_bdds;
+    int32_t k;
+    int32_t jit;
+    int32_t c_lo, c_n;
+    int32_t v_lo, v_n;
+    int32_t cv_row;     // first row of its first tile's block in InstDev::cv
+    int32_t pad[2];
+};
+
+// Per pattern, 8 x 32 words for pairs of layers and lanes: for each of the two
+// layers (low half first) the byte offset, within the tile's multipliers, of
+// the slot's variable's other copy, FDOG_PAIR_ONE if it has none and
+// FDOG_PAIR_REST for a slot that is not tile-local.  Then, per pattern, a word:
+// FDOG_PAIR_PLAIN and the set of tile-local layers if every layer holds 32
+// slots with another copy, or none that is tile-local; else 0.
+#define FDOG_PAIR_REST 0xFFFFu
+#define FDOG_PAIR_ONE 0xFFFEu
+#define FDOG_PAIR_PLAIN 0x80000000u
+
+struct BulkArgs {
+    const InstDev* inst;
+    const uint32_t* pairs;
+    int32_t n_pat;
+    int32_t total;          // tiles of the class
+    int32_t rows;           // rows of 32 floats of one stage: most rows a tile takes
+    int32_t stages;         // tiles a warp has on their way or in work
+};
+
+// shared-memory rows of a warp: its stages, a table of 32 tiles, the terms of four tiles and its barriers
+#define FDOG_BULK_WARP_ROWS(stages, rows) ((stages) * (rows) + 9)
+
 // </jit-abi>
 constexpr int kLbRing = FDOG_LB_RING;
+constexpr int kEpiMaxK = FDOG_EPI_LAYERS;
 
 // ---------------------------------------------------------------------------
 // host-side decomposition
@@ -231,6 +280,11 @@ struct Decomposition {
     std::vector<uint16_t> tpl;
     int64_t n_bdds = 0, n_slots = 0, n_nodes = 0, slots_pad = 0;
     int64_t n_work = 0, n_wpos = 0, n_local_ent = 0;  // sizes of work, wpos, local_ent
+    // bulk sweeps (plan_bulk); empty: none
+    std::vector<BulkRun> bulk_runs;
+    std::vector<uint32_t> bulk_pairs;
+    int32_t bulk_rows = 0;
+    int64_t bulk_cv_rows = 0;
     int kmax[kNumClasses] = {0};
     int nodes_max[kNumClasses] = {0};  // most nodes of a shape of the class
     // Plan built on the device: var, csr_off, csr_pos, work, wpos, local_ent
@@ -328,6 +382,12 @@ int build_decomposition(int32_t n_vars, const double* cost, int32_t n_rows, cons
                         int jit_mode, bool fuse_local, Decomposition& out, std::string& err,
                         const uint8_t* shared = nullptr);
 
+// Whether the instance's shape-specialised tiles can run as bulk sweeps, by
+// its plan alone, and then their plan, from the patterns' entries (which a
+// device-built plan does not hold on the host).
+bool bulk_possible(const Decomposition& d);
+void plan_bulk(Decomposition& d, const uint16_t* local_ent);
+
 // The schedule of the serial update (Eq. 4) on a built decomposition: a
 // variable's ascending level is one more than the largest level of the
 // variables before it in its BDDs (0 if it leads each of them), so variables
@@ -339,6 +399,7 @@ void build_serial_schedule(int32_t n_vars, Decomposition& d);
 int jit_register_shape(const HostShape& s);  // id of the shape's structure
 struct JitKernels {
     const void* fn[4] = {nullptr, nullptr, nullptr, nullptr};  // per sweep mode
+    const void* bulk[2] = {nullptr, nullptr};                  // bulk sweeps: ascending, descending pass
 };
 // host-only NVRTC compile of the module for the given shape ids (cached)
 int jit_compile(const std::vector<int>& ids, std::string& err);

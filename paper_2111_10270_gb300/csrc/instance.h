@@ -41,6 +41,9 @@ struct DevArrays {
     int32_t* csr_pos = nullptr;
     int32_t* patterns = nullptr;
     uint16_t* local_ent = nullptr;
+    float* cv = nullptr;             // bulk sweeps: targets and ids of every tile, places of tile-local copies, runs
+    uint32_t* bulk_pairs = nullptr;
+    BulkRun* bulk_runs = nullptr;
     int32_t* work = nullptr;
     int32_t* wpos = nullptr;
     float* lab = nullptr;            // serial update: labels of every layer and the running labels, per tile
@@ -108,6 +111,8 @@ struct fdog_instance {
     // host-side view of the dual state
     bool pending_T = false;  // deferred differences of the last pass not yet added back
     bool iterated = false;   // iterations ran since the last add-back (running bound available)
+    bool terms_stale = false;  // bulk sweeps ran: T lacks the terms of tile-local variables (flush_terms)
+    bool bulk_off = false;     // no bulk sweeps (the server's views change with every admission)
 
     // rounding result
     bool has_solution = false;
@@ -141,6 +146,14 @@ int fail_cuda(fdog_instance* inst, cudaError_t e, const char* where);
 cudaError_t copy_async(fdog_instance* inst, void* dst, const void* src, size_t bytes, cudaMemcpyKind kind);
 int read_ctl(fdog_instance* inst, InstCtl& out);
 int addback(fdog_instance* inst);
+// bulk sweeps (bulk.cu): whether the instance may use them, and their set-up at build
+inline bool bulk_wanted(const fdog_instance* inst) {
+    return !inst->bulk_off && inst->params.block_threads == 0 && inst->params.update == 0 && !inst->shard;
+}
+int setup_bulk(fdog_instance* inst);
+// stores the tile-local terms that bulk sweeps of any of these instances (the members of b) left out of T
+cudaError_t flush_terms(const std::vector<fdog_instance*>& members, const DevBatch& b, const LaunchCfg& cfg,
+                        cudaStream_t s);
 // shards of a split instance (shard.cu): the copy counts given at set-up
 // against the plan, and the initial multipliers of the shared variables
 int shard_check_copies(fdog_instance* inst);

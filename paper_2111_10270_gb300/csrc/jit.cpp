@@ -119,7 +119,8 @@ std::string nm(const char* p, int t, int v) { return std::string(p) + std::to_st
 std::string nm(const char* p, int t) { return std::string(p) + std::to_string(t); }
 
 // Emits shp_<id>_<mode>(I, base, valid, flags) -> this BDD's share of the bound.
-void emit_shape(std::ostringstream& o, const HostShape& s, int id, int mode) {
+// With bulk (update passes): shb_<id>_<mode>, which reads the tile from the warp's stage in shared memory.
+void emit_shape(std::ostringstream& o, const HostShape& s, int id, int mode, bool bulk = false) {
     const int k = s.k;
     auto width = [&](int t) { return s.lstart[t + 1] - s.lstart[t]; };
     // successor of node v (local) of layer t through arc beta: -1 TOP, -2 BOT, else local index in layer t+1
@@ -127,19 +128,45 @@ void emit_shape(std::ostringstream& o, const HostShape& s, int id, int mode) {
         const int x = beta ? s.hi[s.lstart[t] + v] : s.lo[s.lstart[t] + v];
         return x >= 0 ? x - s.lstart[t + 1] : x;
     };
-    o << "__device__ __forceinline__ float shp_" << id << "_" << mode
-      << "(const InstDev* __restrict__ I, long long base, bool valid, int flags, bool local, float* ep_lam, "
-         "int* ep_var) {\n";
-    o << "  (void)local; (void)ep_lam; (void)ep_var;\n";
-    o << "  float* __restrict__ lam = I->lam;\n  const float omega = I->omega;\n  (void)omega; (void)flags;\n";
-    for (int t = 0; t < k; ++t) o << "  float " << nm("l", t) << " = 0.f, " << nm("u", t) << " = 0.f;\n";
-    o << "  if (valid) {\n";
-    for (int t = 0; t < k; ++t) o << "    " << nm("l", t) << " = lam[base + " << 32 * t << "];\n";
-    if (mode <= 1)
+    if (bulk) {
+        o << "__device__ __forceinline__ float shb_" << id << "_" << mode
+          << "(float* __restrict__ lam, const float* T, bool valid, float omega, bool zero, unsigned plain, "
+             "const float* sl, const float* sc, const int* sv, const unsigned (&pk)[8], int lane) {\n";
+        // sl: the tile's multipliers; sc, sv: rows of targets and ids, addressed as if layer 0 were the first
         for (int t = 0; t < k; ++t)
-            o << "    { const int v = __ldcs(I->var + base + " << 32 * t << "); " << nm("u", t)
-              << " = I->T[v]; if (local) ep_var[" << 32 * t << "] = v; }\n";
-    o << "  }\n";
+            o << "  float " << nm("l", t) << " = sl[" << 32 * t << " + lane], " << nm("u", t) << " = 0.f;\n";
+        for (int t = 0; t < k; ++t)
+            o << "  const unsigned " << nm("p", t) << " = pk[" << t / 2 << (t % 2 ? "] >> 16;\n" : "] & 0xFFFFu;\n");
+        // gathered terms first: they take longest
+        o << "  if (plain) {\n";
+        for (int t = 0; t < k; ++t)
+            o << "    if (!(plain >> " << t << " & 1u)) " << nm("u", t) << " = T[sv[" << 32 * t << " + lane]];\n";
+        for (int t = 0; t < k; ++t)
+            o << "    if (plain >> " << t << " & 1u) " << nm("u", t) << " = (sc[" << 32 * t << " + lane] - ((0.f + "
+              << nm("l", t) << ") + fdog_at(sl, " << nm("p", t) << "))) * 0.5f;\n";
+        o << "  } else {\n";
+        for (int t = 0; t < k; ++t)
+            o << "    if (" << nm("p", t) << " == FDOG_PAIR_REST && valid) " << nm("u", t) << " = T[sv[" << 32 * t
+              << " + lane]];\n";
+        for (int t = 0; t < k; ++t)
+            o << "    if (" << nm("p", t) << " != FDOG_PAIR_REST) " << nm("u", t) << " = fdog_pair_term(sc[" << 32 * t
+              << " + lane], " << nm("l", t) << ", " << nm("p", t) << ", zero, sl);\n";
+        o << "  }\n";
+    } else {
+        o << "__device__ __forceinline__ float shp_" << id << "_" << mode
+          << "(const InstDev* __restrict__ I, long long base, bool valid, int flags, bool local, float* ep_lam, "
+             "int* ep_var) {\n";
+        o << "  (void)local; (void)ep_lam; (void)ep_var;\n";
+        o << "  float* __restrict__ lam = I->lam;\n  const float omega = I->omega;\n  (void)omega; (void)flags;\n";
+        for (int t = 0; t < k; ++t) o << "  float " << nm("l", t) << " = 0.f, " << nm("u", t) << " = 0.f;\n";
+        o << "  if (valid) {\n";
+        for (int t = 0; t < k; ++t) o << "    " << nm("l", t) << " = lam[base + " << 32 * t << "];\n";
+        if (mode <= 1)
+            for (int t = 0; t < k; ++t)
+                o << "    { const int v = __ldcs(I->var + base + " << 32 * t << "); " << nm("u", t)
+                  << " = I->T[v]; if (local) ep_var[" << 32 * t << "] = v; }\n";
+        o << "  }\n";
+    }
 
     // b<t>_<v> = SP(node, TOP) at the current multipliers for layers [from, k)
     auto emit_backward_labels = [&](int from) {
@@ -232,10 +259,14 @@ void emit_shape(std::ostringstream& o, const HostShape& s, int id, int mode) {
     }
     if (mode <= 1) {
         o << "  if (valid) {\n";
-        for (int t = 0; t < k; ++t) o << "    lam[base + " << 32 * t << "] = " << nm("l", t) << ";\n";
-        o << "  }\n  if (local) {\n";
-        for (int t = 0; t < k; ++t) o << "    ep_lam[" << 32 * t << "] = " << nm("l", t) << ";\n";
+        for (int t = 0; t < k; ++t)
+            o << "    lam[" << (bulk ? "" : "base + ") << 32 * t << "] = " << nm("l", t) << ";\n";
         o << "  }\n";
+        if (!bulk) {
+            o << "  if (local) {\n";
+            for (int t = 0; t < k; ++t) o << "    ep_lam[" << 32 * t << "] = " << nm("l", t) << ";\n";
+            o << "  }\n";
+        }
     }
     o << "  return term;\n}\n\n";
 }
@@ -248,12 +279,29 @@ std::string generate_module(const std::vector<int>& ids) {
     o << kJitAbi << "\n";
     for (int id : ids)
         for (int mode = 0; mode < 4; ++mode) emit_shape(o, g_shapes[id], id, mode);
+    // multiplier at a byte offset of the tile; deferred term of a tile-local slot, as in fdog_tile_local_sums
+    o << "__device__ __forceinline__ float fdog_at(const float* sl, unsigned p) {\n"
+         "  return *(const float*)((const char*)sl + p);\n}\n"
+         "__device__ __forceinline__ float fdog_pair_term(float C, float l, unsigned p, bool zero, const float* sl) {\n"
+         "  float s = 0.f + l, inv = 1.f;\n"
+         "  if (p != FDOG_PAIR_ONE) { s += fdog_at(sl, p); inv = 0.5f; }\n"
+         "  return zero ? 0.f : (C - s) * inv;\n}\n\n";
+    for (int id : ids)
+        for (int mode = 0; mode < 2; ++mode) emit_shape(o, g_shapes[id], id, mode, true);
     o << "#define FDOG_DISPATCH(MODE) \\\n";
     for (int mode = 0; mode < 4; ++mode) {
         o << "  " << (mode ? "else " : "") << "if (MODE == " << mode << ") { switch (jit) { \\\n";
         for (int id : ids)
             o << "    case " << id << ": term = shp_" << id << "_" << mode
               << "(I, base, valid, a.flags, local, ep_lam + lane, ep_var + lane); break; \\\n";
+        o << "    default: break; } } \\\n";
+    }
+    o << "\n#define FDOG_BULK_DISPATCH(MODE) \\\n";
+    for (int mode = 0; mode < 2; ++mode) {
+        o << "  " << (mode ? "else " : "") << "if (MODE == " << mode << ") { switch (jit) { \\\n";
+        for (int id : ids)
+            o << "    case " << id << ": term = shb_" << id << "_" << mode
+              << "(lam, T, valid, omega, zero, plain, sl, sc, sv, pk, lane); break; \\\n";
         o << "    default: break; } } \\\n";
     }
     o << "\n" << kJitSkeleton;
@@ -303,9 +351,10 @@ int jit_kernels(const std::vector<int>& ids_in, JitKernels& out, std::string& er
         err = std::string("cudaLibraryLoadData: ") + cudaGetErrorString(e);
         return FDOG_ECUDA;
     }
-    const char* names[4] = {"fdog_jit_fwd", "fdog_jit_bwd", "fdog_jit_mm", "fdog_jit_eval"};
+    const char* names[6] = {"fdog_jit_fwd", "fdog_jit_bwd", "fdog_jit_mm", "fdog_jit_eval", "fdog_bulk_fwd",
+                            "fdog_bulk_bwd"};
     JitKernels kk;
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < 6; ++m) {
         cudaKernel_t kern = nullptr;
         e = cudaLibraryGetKernel(&kern, lib, names[m]);
         if (e != cudaSuccess) {
@@ -313,7 +362,7 @@ int jit_kernels(const std::vector<int>& ids_in, JitKernels& out, std::string& er
             err = std::string("cudaLibraryGetKernel: ") + cudaGetErrorString(e);
             return FDOG_ECUDA;
         }
-        kk.fn[m] = reinterpret_cast<const void*>(kern);
+        (m < 4 ? kk.fn[m] : kk.bulk[m - 4]) = reinterpret_cast<const void*>(kern);
     }
     g_modules.emplace(key, kk);  // the library stays loaded for the life of the process
     out = kk;

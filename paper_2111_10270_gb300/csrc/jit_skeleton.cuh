@@ -110,3 +110,194 @@ extern "C" __global__ void __launch_bounds__(256) fdog_jit_fwd(SweepArgs a) { fd
 extern "C" __global__ void __launch_bounds__(256) fdog_jit_bwd(SweepArgs a) { fdog_jit_sweep<1>(a); }
 extern "C" __global__ void __launch_bounds__(256) fdog_jit_mm(SweepArgs a) { fdog_jit_sweep<2>(a); }
 extern "C" __global__ void __launch_bounds__(256) fdog_jit_eval(SweepArgs a) { fdog_jit_sweep<3>(a); }
+
+// ---- bulk sweeps -------------------------------------------------------------
+// Update passes of one large instance.  In the sweeps above a warp waits in
+// turn for its tile's descriptor, its multipliers and ids, the terms they
+// name, and at the end for the targets C of its tile-local variables; with
+// every warp slot of the GPU taken they run at 62 and 70 us a pass on the
+// 512x512 grid with four labels, for 374 MB, and no part of that chain can be
+// moved forward because registers are all in use.  Here the warps stay and
+// walk many tiles each, and what a tile reads is copied ahead into shared
+// memory by bulk copies (cp.async.bulk, one mbarrier per stage of a warp),
+// which hold no registers:
+//   * its multipliers, one run of k rows;
+//   * one block with the targets of its layers with tile-local slots, in slot
+//     order (so a variable's target is there for each of its copies), and the
+//     ids of its other layers.
+// The term of a tile-local variable (all of whose at most two copies lie in
+// the tile) is formed here, from the multipliers the last pass left in the
+// tile, instead of at the end of that pass: T is neither written nor gathered
+// for it, and its slots need no ids.  The same FP32 operations in the same
+// order, so the same terms.  A pass moves 274 MB, in about 48 us: the 500
+// iterations and two roundings of that grid went from 88.2 to 69.5 ms.  What
+// bounds it now is instructions, 281 and 304 a tile with 68% of the issue
+// slots taken (338 before tiles were looked up 16 at a time, the second copy
+// was merged, and plain patterns got a path without choices per slot).  Two
+// stages (69.5 ms; three 70.3, four 74.5): at 62 registers four blocks of eight
+// warps fit an SM, and more stages take L1 from the gathers of T.  Capping the
+// registers at 48 for a fifth block made them spill (74.9 ms).  The L2 window
+// on T is worth 1 ms.
+__device__ __forceinline__ unsigned fdog_smem_addr(const void* p) {
+    return (unsigned)__cvta_generic_to_shared(p);
+}
+
+// waits for a stage's copies; gives up (false) after a second
+__device__ __forceinline__ bool fdog_bulk_wait(unsigned bar, unsigned parity) {
+    unsigned long long t0 = 0, t;
+    for (;;) {
+        unsigned done;
+        asm volatile(
+            "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > 1000000000ull) return false;
+    }
+}
+
+__device__ __forceinline__ void fdog_bulk_copy(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
+// (s, c) <- (s, c) + (x, y) for compensated FP32 pairs, as the butterflies above form them
+__device__ __forceinline__ void fdog_pair_add(float& s, float& c, float x, float y) {
+    const float sum = s + x;
+    const float bp = sum - s;
+    const float err = (s - (sum - bp)) + (x - bp);
+    s = sum;
+    c = c + y + err;
+}
+
+template <int MODE>
+__device__ __forceinline__ void fdog_bulk_sweep(const BulkArgs& a) {
+    extern __shared__ __align__(128) float fdog_stages[];
+    const int lane = threadIdx.x & 31;
+    const int wpb = blockDim.x >> 5;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // this warp's rows: stages; a table of the 32 tiles around the current one (16 ahead are filled in at a time, a
+    // lane per tile, so that finding a tile costs next to nothing); the terms of four tiles; the barriers
+    float* const stage0 = fdog_stages + (threadIdx.x >> 5) * FDOG_BULK_WARP_ROWS(a.stages, a.rows) * 32;
+    int4* const tab = (int4*)(stage0 + a.stages * a.rows * 32);
+    float* const terms = (float*)(tab + 32);
+    const unsigned bars = fdog_smem_addr(terms + 136);
+    if (lane == 0) {
+        for (int s = 0; s < a.stages; ++s)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * s) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("fence.proxy.async.global;" ::: "memory");  // the copies read what kernels wrote
+    const InstDev* __restrict__ I = a.inst;
+    InstCtl* const ctl = I->ctl;
+    if (FDOG_INACTIVE(ctl)) return;
+    const bool zero = MODE == 0 && ctl->t_zero;  // a descending pass follows an ascending one
+    const float omega = I->omega;
+    float* const lam0 = I->lam;
+    const float* const cv0 = I->cv;
+    const float* const T = I->T;
+    const int first = I->bulk_first;
+    const int stride = gridDim.x * wpb;
+    const int g0 = blockIdx.x * wpb + (threadIdx.x >> 5);
+    const int n = g0 < a.total ? (a.total - g0 + stride - 1) / stride : 0;  // tiles of this warp
+
+    auto fill = [&](int block) {
+        const int it = 16 * block + lane;
+        if (lane < 16 && it < n) {
+            const int g = g0 + it * stride;
+            const BulkRun* r = I->bulk_runs;
+            for (int q = I->n_bulk_runs - 1; q > 0; --q)
+                if (I->bulk_runs[q].tile <= g) {
+                    r = I->bulk_runs + q;
+                    break;
+                }
+            const int j = g - r->tile;
+            const int n_valid = min(32, r->n_bdds - 32 * j);
+            tab[it & 31] = make_int4(r->slot_base + j * r->k * 32, r->cv_row + j * (r->c_n + r->v_n),
+                                     r->k | r->c_n << 5 | r->v_n << 10 | r->c_lo << 15 | r->v_lo << 19 | n_valid << 23,
+                                     r->jit << 8 | (I->tiles[first + g].pattern + 1));
+        }
+        __syncwarp();
+    };
+    auto issue = [&](int it, int s) {
+        if (it < n && lane == 0) {
+            const int4 e = tab[it & 31];
+            const unsigned rows = e.z & 31, more = (e.z >> 5 & 31) + (e.z >> 10 & 31);
+            const unsigned bar = bars + 8u * s;
+            const unsigned dst = fdog_smem_addr(stage0 + s * a.rows * 32);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((rows + more) * 128u)
+                         : "memory");
+            fdog_bulk_copy(dst, lam0 + e.x, rows * 128u, bar);
+            fdog_bulk_copy(dst + rows * 128u, cv0 + e.y * 32, more * 128u, bar);
+        }
+    };
+    fill(0);
+    for (int s = 0; s < a.stages; ++s) issue(s, s);
+    unsigned pk[8], plain_of = 0;
+    int have = -1, s = 0;
+    unsigned parity = 0;
+    bool late = false;
+    for (int i = 0; i < n; ++i) {
+        if ((i & 15) == 0) fill((i >> 4) + 1);
+        const int4 e = tab[i & 31];
+        const int pat = e.w & 255;
+        if (pat != have) {  // most neighbouring tiles have the same pattern
+            have = pat;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                pk[q] = pat > 0 ? __ldg(a.pairs + ((pat - 1) * 8 + q) * 32 + lane) : 0xFFFFFFFFu;
+            plain_of = pat > 0 ? __ldg(a.pairs + a.n_pat * 256 + pat - 1) : FDOG_PAIR_PLAIN;
+        }
+        const int k = e.z & 31, n_valid = e.z >> 23;
+        const unsigned plain = n_valid == 32 && !zero ? plain_of : 0u;
+        const int jit = e.w >> 8;
+        const bool valid = lane < n_valid;
+        float* const lam = lam0 + (e.x + lane);
+        const float* const sl = stage0 + s * a.rows * 32;
+        const float* const sc = sl + (k - (e.z >> 15 & 15)) * 32;
+        const int* const sv = (const int*)(sl + (k + (e.z >> 5 & 31) - (e.z >> 19 & 15)) * 32);
+        // a lane that has waited in vain reports it (the host then returns an error) and waits no more; every lane
+        // goes on, so that the warp stays together
+        if (!late && !fdog_bulk_wait(bars + 8u * s, parity)) {
+            late = true;
+            ctl->error = 1;
+        }
+        float term = 0.f;
+        FDOG_BULK_DISPATCH(MODE)
+        __syncwarp();  // every lane has read the stage
+        issue(i + a.stages, s);
+        if (++s == a.stages) {
+            s = 0;
+            parity ^= 1u;
+        }
+        if (MODE == 1) {
+            // Partials of the bound, four tiles at a time: eight lanes reduce one tile, in the order of the
+            // butterflies above (lane l + 16, l + 8, then 4, 2, 1).  A butterfly per tile took 45 instructions,
+            // this takes 16.
+            terms[(i & 3) * 33 + lane] = valid ? term : 0.f;
+            if ((i & 3) == 3 || i == n - 1) {
+                __syncwarp();
+                const int q = lane >> 3, j = lane & 7;
+                const float* const t = terms + q * 33 + j;
+                float x = t[0], xc = 0.f, y = t[8], yc = 0.f;
+                fdog_pair_add(x, xc, t[16], 0.f);
+                fdog_pair_add(y, yc, t[24], 0.f);
+                fdog_pair_add(x, xc, y, yc);
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) {
+                    const float o = __shfl_xor_sync(FDOG_FULL, x, off);
+                    const float oc = __shfl_xor_sync(FDOG_FULL, xc, off);
+                    fdog_pair_add(x, xc, o, oc);
+                }
+                if (j == 0 && q <= (i & 3)) I->tile_lb[first + g0 + (i - (i & 3) + q) * stride] = make_float2(x, xc);
+                __syncwarp();
+            }
+        }
+    }
+}
+
+extern "C" __global__ void __launch_bounds__(256) fdog_bulk_fwd(BulkArgs a) { fdog_bulk_sweep<0>(a); }
+extern "C" __global__ void __launch_bounds__(256) fdog_bulk_bwd(BulkArgs a) { fdog_bulk_sweep<1>(a); }

@@ -78,6 +78,7 @@ __device__ __forceinline__ void lb_reduce_block(const LbArgs& a, int g, bool com
     if (threadIdx.x == 0) {
         if (n_chunks > kLbFew) ctl->ticket = 0;
         if (commit) {
+            ctl->t_zero = 0;
             commit_iteration(ctl, lb, in);
         } else {
             ctl->lb_staged = lb;
@@ -180,7 +181,34 @@ __global__ void __launch_bounds__(256) zero_T_kernel(FlatArgs a) {
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < a.total; g += gridDim.x * blockDim.x) {
         const int ii = find_inst(a.prefix, a.n_inst, g);
         const InstDev* __restrict__ I = a.insts + ii;
-        I->T[g - __ldg(a.prefix + ii)] = 0.f;
+        const int i = g - __ldg(a.prefix + ii);
+        I->T[i] = 0.f;
+        if (i == 0) I->ctl->t_zero = 1;
+    }
+}
+
+// The pending terms of the tile-local variables into T (a warp per tile; FP32
+// operations and order as in tile_local_sums).
+__global__ void __launch_bounds__(256) local_terms_kernel(FlatArgs a) {
+    const int lane = threadIdx.x & 31;
+    const int warps = (gridDim.x * blockDim.x) >> 5;
+    for (int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < a.total; g += warps) {
+        const int ii = find_inst(a.prefix, a.n_inst, g);
+        const InstDev* __restrict__ I = a.insts + ii;
+        const TileDev tile = I->tiles[g - __ldg(a.prefix + ii)];
+        if (tile.pattern < 0 || I->ctl->t_zero) continue;  // T holds zeros
+        const int2 pat = reinterpret_cast<const int2*>(I->patterns)[tile.pattern];
+        const float* __restrict__ lam = I->lam + tile.slot_base;
+        for (int e = lane; e < pat.y; e += kTile) {
+            const ushort4 o = reinterpret_cast<const ushort4*>(I->local_ent)[pat.x + e];
+            float s = 0.f + lam[o.x];
+            int c = 1;
+            if (o.y != 0xFFFFu) { s += lam[o.y]; ++c; }
+            if (o.z != 0xFFFFu) { s += lam[o.z]; ++c; }
+            if (o.w != 0xFFFFu) { s += lam[o.w]; ++c; }
+            const int v = I->var[tile.slot_base + o.x];
+            I->T[v] = (I->C[v] - s) * dev::inv_copies(c);
+        }
     }
 }
 
@@ -469,7 +497,9 @@ cudaError_t launch_class(const DevBatch& b, int cls, int mode, int mm_flags, con
     // update passes of the dominant class keep the deferred terms they gather in L2
     const L2Window l2 = dominant && (mode == kFwdUpdate || mode == kBwdUpdate) ? b.l2 : L2Window();
     cudaError_t e;
-    if (cls == kJitClass) {
+    if (cls == kJitClass && (mode == kFwdUpdate || mode == kBwdUpdate) && b.bulk.ready) {
+        e = launch_bulk(b, mode, cfg, s);
+    } else if (cls == kJitClass) {
         void* kargs[] = {&args};
         e = cudaSuccess;
         if (smem > 48 * 1024)
@@ -688,6 +718,14 @@ cudaError_t launch_lb_reduce(const DevBatch& b, int target, const LaunchCfg& cfg
                            L2Window());
 }
 
+cudaError_t launch_local_terms(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s) {
+    if (b.tiles_all_total == 0) return cudaSuccess;
+    cfg.count();
+    local_terms_kernel<<<blocks_for(b.tiles_all_total, 8, cfg.num_sms * 8), 256, 0, s>>>(
+        flat(b, b.tile_all_prefix, b.tiles_all_total));
+    return cudaGetLastError();
+}
+
 cudaError_t launch_init(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s) {
     cfg.count((b.vars_total > 0) + (b.slots_total > 0));
     if (b.vars_total > 0)
@@ -696,7 +734,8 @@ cudaError_t launch_init(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s)
     if (b.slots_total > 0)
         init_lam_kernel<<<blocks_for(b.slots_total, 256, cfg.num_sms * 8), 256, 0, s>>>(
             flat(b, b.slot_prefix, b.slots_total));
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_bulk_targets(b, cfg, s);
 }
 
 cudaError_t launch_addback(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s) {
@@ -732,7 +771,8 @@ cudaError_t launch_round_apply(const DevBatch& b, const LaunchCfg& cfg, cudaStre
     const int wide_blocks = (b.wide_total + 7) / 8;
     round_apply_kernel<<<wide_blocks + blocks_for(b.vars_total, 256, cfg.num_sms * 8), 256, 0, s>>>(
         flat(b, b.var_prefix, b.vars_total), flat(b, b.wide_prefix, b.wide_total), wide_blocks);
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_bulk_targets(b, cfg, s);
 }
 
 cudaError_t launch_objective(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s) {

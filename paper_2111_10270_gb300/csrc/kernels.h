@@ -54,9 +54,22 @@ struct L2Window {
 // device maximum; never lowered) and returns the window for [base, base + bytes).
 L2Window l2_window_for(int device, void* base, size_t bytes);
 
+// a kernel launch with programmatic stream serialization (the kernel calls
+// pdl_wait before it touches memory) and an optional L2 access-policy window
+// (kernels.cu)
+cudaError_t launch_windowed(const void* fn, int blocks, int threads, void** args, size_t smem, cudaStream_t s,
+                            const L2Window& l2);
+
 struct FlatArgsS {
     const InstDev* I;
     int32_t total;
+};
+
+// Bulk sweeps of one instance (bulk.cu).
+struct BulkPlan {
+    bool ready = false;
+    BulkArgs args{};
+    int blocks_per_sm = 0;
 };
 
 struct DevBatch {
@@ -85,6 +98,8 @@ struct DevBatch {
     JitKernels jit;                          // kernels of the shape-specialised class
     SerialPlan serial;                       // serial update only
     L2Window l2;                             // update sweeps of a one-instance batch: its T array
+    BulkPlan bulk;                           // bulk sweeps of a one-instance batch (if ready)
+    bool any_cv = false;                     // some member has bulk sweeps
 };
 
 
@@ -142,6 +157,12 @@ cudaError_t launch_eval64(const DevBatch& b, bool add_t, const LaunchCfg& cfg, c
 cudaError_t launch_init(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s);
 cudaError_t launch_addback(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s);
 cudaError_t launch_zero_T(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s);
+// one update pass of the shape-specialised class as a bulk sweep (bulk.cu)
+cudaError_t launch_bulk(const DevBatch& b, int mode, const LaunchCfg& cfg, cudaStream_t s);
+// the pending terms of the tile-local variables into T, which the bulk sweeps leave out
+cudaError_t launch_local_terms(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s);
+// InstDev::cv from C, after every change of C
+cudaError_t launch_bulk_targets(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s);
 cudaError_t launch_round_test(const DevBatch& b, const LaunchCfg& cfg, cudaStream_t s);
 
 // per-instance control-block operations (instance_op_kernel)

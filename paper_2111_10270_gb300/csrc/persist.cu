@@ -137,7 +137,10 @@ __global__ void __launch_bounds__(kPersistThreads, 2) persist_iterations_kernel(
             const InstDev* __restrict__ I = a.lb.insts + ii;
             if (__ldg(a.lb.prefix + ii + 1) == __ldg(a.lb.prefix + ii) || FDOG_INACTIVE(I->ctl)) continue;
             const double v = lb_total(I, ss, sc);
-            if (threadIdx.x == 0) commit_iteration(I->ctl, v, commit_in(I->ctl));
+            if (threadIdx.x == 0) {
+                I->ctl->t_zero = 0;
+                commit_iteration(I->ctl, v, commit_in(I->ctl));
+            }
             __syncthreads();
         }
         ok = grid_barrier(a);

@@ -839,6 +839,12 @@ int plan_on_device(fdog_instance* inst, int jit_mode, bool fuse_local) {
                                                       out.d_wpos);
     PLAN_CHECK(cudaGetLastError());
     PLAN_CHECK(cudaStreamSynchronize(st));
+    if (bulk_wanted(inst) && bulk_possible(out)) {
+        std::vector<uint16_t> ent(static_cast<size_t>(out.n_local_ent));
+        PLAN_CHECK(cudaMemcpyAsync(ent.data(), out.d_local_ent, sizeof(uint16_t) * ent.size(), cudaMemcpyDeviceToHost, st));
+        PLAN_CHECK(cudaStreamSynchronize(st));
+        plan_bulk(out, ent.data());
+    }
     out.on_device = true;
     inst->plan_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     return FDOG_OK;

@@ -269,6 +269,7 @@ int fdog_server_submit(fdog_server* s, fdog_instance* inst, uint64_t* ticket) {
     Job* j = new (std::nothrow) Job();
     if (!j) return FDOG_ENOMEM;
     j->inst = inst;
+    inst->bulk_off = true;
     if (!inst->planned && inst->params.planner != 1) {
         // planned by the worker at admission, on the device where the builder takes it
         j->plan_on_admit = true;
@@ -365,6 +366,7 @@ int fdog_server_take(fdog_server* s, uint64_t ticket, fdog_instance** out) {
     Job* j = it->second;
     if (j->state != 2) return FDOG_ESTATE;
     *out = j->inst;
+    j->inst->bulk_off = false;
     s->jobs.erase(it);
     delete j;
     return FDOG_OK;

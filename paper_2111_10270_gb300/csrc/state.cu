@@ -66,11 +66,14 @@ int fdog_export_state(fdog_instance* inst, void* buf, size_t* bytes) {
     h.n_tiles = static_cast<int64_t>(inst->dec.tiles.size());
     h.layout_hash = layout_hash(inst);
     h.omega = inst->params.omega;
+    // every pending term into T
+    cudaError_t e = flush_terms({inst}, inst->batch, inst->cfg, inst->stream);
     char* out = static_cast<char*>(buf);
     std::memcpy(out, &h, sizeof(h));
     size_t off = sizeof(h);
     cudaStream_t s = inst->stream;
-    cudaError_t e = copy_async(inst, out + off, inst->dev.lam, sizeof(float) * h.slots_pad, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess)
+        e = copy_async(inst, out + off, inst->dev.lam, sizeof(float) * h.slots_pad, cudaMemcpyDeviceToHost);
     off += sizeof(float) * h.slots_pad;
     if (e == cudaSuccess) e = copy_async(inst, out + off, inst->dev.T, sizeof(float) * h.n_vars, cudaMemcpyDeviceToHost);
     off += sizeof(float) * h.n_vars;
@@ -80,6 +83,9 @@ int fdog_export_state(fdog_instance* inst, void* buf, size_t* bytes) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (prev >= 0 && prev != inst->device) cudaSetDevice(prev);
     if (e != cudaSuccess) return fail_cuda(inst, e, "export state");
+    // whether T is zero follows from the flags and the update mode: not part of the format
+    const int32_t none = 0;
+    std::memcpy(out + off + offsetof(InstCtl, t_zero), &none, sizeof(none));
     *bytes = need;
     return FDOG_OK;
 }
@@ -109,10 +115,16 @@ int fdog_import_state(fdog_instance* inst, const void* buf, size_t bytes) {
     in += sizeof(float) * h.n_vars;
     if (e == cudaSuccess) e = copy_async(inst, inst->dev.C, in, sizeof(float) * h.n_vars, cudaMemcpyHostToDevice);
     in += sizeof(float) * h.n_vars;
-    if (e == cudaSuccess) e = copy_async(inst, inst->dev.ctl, in, sizeof(InstCtl), cudaMemcpyHostToDevice);
+    InstCtl ctl;
+    std::memcpy(&ctl, in, sizeof(ctl));
+    // the serial update keeps no deferred terms
+    ctl.t_zero = (h.flags & 1u) == 0 || inst->params.update == 1 ? 1 : 0;
+    if (e == cudaSuccess) e = copy_async(inst, inst->dev.ctl, &ctl, sizeof(InstCtl), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = launch_bulk_targets(inst->batch, inst->cfg, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (prev >= 0 && prev != inst->device) cudaSetDevice(prev);
     if (e != cudaSuccess) return fail_cuda(inst, e, "import state");
+    inst->terms_stale = false;
     inst->pending_T = (h.flags & 1u) != 0;
     inst->iterated = (h.flags & 2u) != 0;
     return FDOG_OK;

@@ -832,12 +832,6 @@ __global__ void __launch_bounds__(256) sweep_seg_kernel(SweepArgs a) {
 
 }  // namespace dev
 
-// a kernel launch with programmatic stream serialization (the kernel calls
-// pdl_wait before it touches memory) and an optional L2 access-policy window
-// (kernels.cu)
-cudaError_t launch_windowed(const void* fn, int blocks, int threads, void** args, size_t smem, cudaStream_t s,
-                            const L2Window& l2);
-
 // host-side dispatch of one width's instantiations (defined in sweep_w<W>.cu)
 template <int W>
 cudaError_t launch_sweep_width(bool reg, int mode, int blocks, int threads, size_t smem, cudaStream_t s,

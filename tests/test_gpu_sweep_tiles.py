@@ -137,3 +137,77 @@ def test_slots_as_listed(P, planner, count):
             blob = inst.export_state()
             inst.release()
             inst.build(0).import_state(blob)
+
+
+def join(*parts):
+    """The ILPs side by side, without common variables."""
+    off = np.cumsum([0] + [p.n_vars for p in parts])
+    ptr = np.concatenate([[0], np.cumsum(np.concatenate([np.diff(p.row_ptr) for p in parts]))])
+    return ilpgen.ILP(int(off[-1]), np.concatenate([p.cost for p in parts]), ptr.astype(np.int64),
+                      np.concatenate([p.col + o for p, o in zip(parts, off)]).astype(np.int32),
+                      np.concatenate([p.coef for p in parts]), np.concatenate([p.sense for p in parts]),
+                      np.concatenate([p.rhs for p in parts]), name="joined")
+
+
+# Instances that run bulk sweeps: grids whose edges fill their tiles (4, 2 and 8 labels), and one of them beside
+# grids whose edges are cut by the tile's end (slots of one layer of both kinds), rows of variables with one copy,
+# partial last tiles and tiles without any local variable.
+BULK = {
+    "4": lambda: ilpgen.mrf_grid(190, 190, 4, 3, potts_max=2.0),
+    "2": lambda: ilpgen.mrf_grid(370, 361, 2, 3, potts_max=2.0),
+    "8": lambda: ilpgen.mrf_grid(131, 133, 8, 3, potts_max=2.0),
+    "mixed": lambda: join(ilpgen.mrf_grid(195, 191, 4, 3), ilpgen.mrf_grid(61, 53, 3, 4), ilpgen.mrf_grid(41, 37, 5, 5),
+                          ilpgen.mrf_grid(29, 31, 7, 6), rows_ilp(*PATTERNS["flow5"], 4111, 7, False),
+                          rows_ilp(*PATTERNS["marg6"], 4099, 8, True)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(BULK))
+def test_bulk_sweeps_match_the_ordinary_ones(P, name):
+    """Every state that can be read, bit for bit as without bulk sweeps (block_threads set: never used)."""
+    g = BULK[name]()
+
+    def make(**kw):
+        return P.Instance.from_ilp(g, P.capi.default_params(tol=0.0, max_rounds=3, jit=1, **kw)).build(0)
+
+    a, b = make(), make(block_threads=128)
+    assert a.info()["device_bytes"] > b.info()["device_bytes"]  # the plan of the bulk sweeps
+
+    def arrays(inst):
+        blob = inst.export_state()
+        assert blob[-4:] == b"\0\0\0\0"
+        return blob[:-CTL_BYTES]
+
+    def same():
+        assert a.lower_bound() == b.lower_bound()
+        assert arrays(a) == arrays(b)
+
+    same()
+    assert a.iterate(1) == b.iterate(1)
+    same()
+    assert a.iterate(9) == b.iterate(9)
+    blob = a.export_state()
+    same()
+    c = make()
+    c.import_state(blob)
+    assert a.iterate(2) == b.iterate(2) == c.iterate(2)
+    assert arrays(a) == arrays(c)
+    for inst in (a, b):
+        inst.finalize()
+    same()
+    assert a.iterate(2) == b.iterate(2)
+    # a batch runs the ordinary sweeps on what the bulk sweeps left
+    small = P.Instance.from_ilp(ilpgen.mrf_grid(9, 9, 3, 1), P.capi.default_params(tol=0.0, max_rounds=3)).build(0)
+    batch = P.Batch([a, small])
+    batch.solve(3)
+    batch.close()
+    b.iterate(3)
+    b.primal_round()
+    same()
+    assert np.array_equal(a.solution()[0], b.solution()[0])
+    assert a.iterate(2) == b.iterate(2)  # perturbed targets
+    same()
+    a.reset(), b.reset()
+    assert a.iterate(4) == b.iterate(4)
+    assert a.primal_round() == b.primal_round()
+    same()
