@@ -12,13 +12,16 @@
 #define FDOG_INF __int_as_float(0x7f800000)
 #define FDOG_FULL 0xffffffffu
 
-__device__ __forceinline__ int fdog_find_inst(const int32_t* __restrict__ prefix, int n, int g) {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(prefix + mid) <= g) lo = mid; else hi = mid - 1;
+// largest instance index i with prefix[i] <= g, g the same in every lane
+__device__ __forceinline__ int fdog_find_inst(const int32_t* __restrict__ prefix, int n, int g, int lane) {
+    if (n == 1) return 0;
+    int at = 0;
+    for (int b = 0; b < n; b += 32) {
+        const unsigned m = __ballot_sync(FDOG_FULL, b + lane < n && __ldg(prefix + b + lane) <= g);
+        at += __popc(m);
+        if (m != FDOG_FULL) break;
     }
-    return lo;
+    return at - 1;
 }
 
 // Deferred terms of the tile-local variables, formed right after an update
@@ -46,7 +49,7 @@ __device__ __forceinline__ void fdog_tile_local_sums(const InstDev* __restrict__
 // computed so that the next tile's first loads hit L2.
 __device__ __forceinline__ void fdog_prefetch_tile(const SweepArgs& a, int g, int lane) {
     if (g >= a.total) return;
-    const int ii = fdog_find_inst(a.prefix, a.n_inst, g);
+    const int ii = fdog_find_inst(a.prefix, a.n_inst, g, lane);
     const InstDev* __restrict__ I = a.insts + ii;
     const TileDev tile = I->tiles[__ldg(a.first + ii) + (g - __ldg(a.prefix + ii))];
     const int k = I->shapes[tile.shape].k;
@@ -73,7 +76,7 @@ __device__ __forceinline__ void fdog_jit_sweep(const SweepArgs& a) {
     int* ep_var = (int*)(ep_lam + (long long)a.epi * 32);
     for (int g = blockIdx.x * wpb + wib; g < a.total; g += gridDim.x * wpb) {
         fdog_prefetch_tile(a, g + gridDim.x * wpb, lane);
-        const int ii = fdog_find_inst(a.prefix, a.n_inst, g);
+        const int ii = fdog_find_inst(a.prefix, a.n_inst, g, lane);
         const InstDev* __restrict__ I = a.insts + ii;
         if (MODE <= 1 && FDOG_INACTIVE(I->ctl)) continue;
         const int ti = __ldg(a.first + ii) + (g - __ldg(a.prefix + ii));

@@ -123,7 +123,12 @@ __global__ void __launch_bounds__(256, 8) deferred_sum_kernel(FlatArgs work, Fla
         return;
     }
     const int g = (blk - wide_blocks) * static_cast<int>(blockDim.x) + static_cast<int>(threadIdx.x);
-    if (g < work.total) reduce_T_one<END>(work, g);
+    // the instance of the warp's first variable, then this thread's (a warp rarely spans two)
+    const int lane = threadIdx.x & 31;
+    int ii = dev::find_inst_warp(work.prefix, work.n_inst, g - lane, lane);
+    if (g >= work.total) return;
+    while (ii + 1 < work.n_inst && __ldg(work.prefix + ii + 1) <= g) ++ii;
+    reduce_T_one<END>(work, g, ii);
 }
 
 // End of an iteration for every member whose bound was staged: ring, counter

@@ -98,7 +98,8 @@ __device__ __forceinline__ void sweep_pass(const SweepArgs (&c)[2], int n_reg, i
 }
 
 __device__ __forceinline__ void deferred_sums(const PersistArgs& a, int gt, int nt, int gw, int nw, int lane) {
-    for (int g = gt; g < a.work.total; g += nt) reduce_T_one(a.work, g);
+    for (int g = gt; g < a.work.total; g += nt)
+        reduce_T_one(a.work, g, find_inst(a.work.prefix, a.work.n_inst, g));
     for (int g = gw; g < a.wide.total; g += nw) reduce_T_wide_one(a.wide, g, lane);
 }
 

@@ -27,15 +27,14 @@ struct FlatArgs {
 // the block scheduler keeps every warp slot busy); its slot positions come
 // from the bucket of its copy count, one coalesced column per copy, so all of
 // its multiplier gathers are issued together.
-// one listed variable with at most 8 copies (work index g of the flat batch).
+// one listed variable with at most 8 copies (work index g of the flat batch, in instance ii).
 // Instances whose stopping rule or iteration limit has stopped them are left
 // alone.  Without SNAPSHOT the test reads the control block and work index 0
 // of each instance records its outcome in InstCtl::pass_active; with SNAPSHOT
 // it reads that record instead of the control block's live state, which the
 // end-of-iteration kernel's commit may change while this runs.
 template <bool SNAPSHOT = false>
-__device__ __forceinline__ void reduce_T_one(const FlatArgs& a, int g) {
-    const int ii = find_inst(a.prefix, a.n_inst, g);
+__device__ __forceinline__ void reduce_T_one(const FlatArgs& a, int g, int ii) {
     const InstDev* __restrict__ I = a.insts + ii;
     const int w = g - __ldg(a.prefix + ii);  // below wb_start[FDOG_WBUCKETS - 1]: at most 8 copies
     if (SNAPSHOT) {
@@ -183,7 +182,7 @@ __device__ __forceinline__ void commit_iteration(InstCtl* ctl, double lb, const 
 // the activity when it is off).
 template <bool SNAPSHOT = false>
 __device__ __forceinline__ void reduce_T_wide_one(const FlatArgs& a, int g, int lane) {
-    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const int ii = find_inst_warp(a.prefix, a.n_inst, g, lane);
     const InstDev* __restrict__ I = a.insts + ii;
     const int w = g - __ldg(a.prefix + ii);
     if (SNAPSHOT) {

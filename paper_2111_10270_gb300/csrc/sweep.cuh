@@ -41,6 +41,19 @@ __device__ __forceinline__ int find_inst(const int32_t* __restrict__ prefix, int
     return lo;
 }
 
+// The same by a whole warp, g the same in every lane: one load for up to 32
+// instances instead of one after the other.
+__device__ __forceinline__ int find_inst_warp(const int32_t* __restrict__ prefix, int n, int g, int lane) {
+    if (n == 1) return 0;
+    int at = 0;
+    for (int b = 0; b < n; b += 32) {
+        const unsigned m = __ballot_sync(kFull, b + lane < n && __ldg(prefix + b + lane) <= g);
+        at += __popc(m);
+        if (m != kFull) break;
+    }
+    return at - 1;
+}
+
 template <int W>
 __device__ __forceinline__ void load_codes(const uint16_t* __restrict__ p, uint32_t (&c)[W]) {
     if constexpr (W == 2) {
@@ -201,7 +214,7 @@ __device__ __forceinline__ void tile_local_sums(const InstDev* __restrict__ I, i
 // computed so that the next tile's first loads hit L2.
 __device__ __forceinline__ void prefetch_tile(const SweepArgs& a, int g, int lane) {
     if (g >= a.total) return;
-    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const int ii = find_inst_warp(a.prefix, a.n_inst, g, lane);
     const InstDev* __restrict__ I = a.insts + ii;
     const TileDev tile = I->tiles[__ldg(a.first + ii) + (g - __ldg(a.prefix + ii))];
     const int k = I->shapes[tile.shape].k;
@@ -251,7 +264,7 @@ template <int W, int MODE>
 __device__ __forceinline__ void reg_tile(const SweepArgs& a, int g, int g_next, float* wsm, int lane) {
     constexpr bool update = MODE == kFwdUpdate || MODE == kBwdUpdate;
     prefetch_tile(a, g_next, lane);
-    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const int ii = find_inst_warp(a.prefix, a.n_inst, g, lane);
     const InstDev* __restrict__ I = a.insts + ii;
     if (update && FDOG_INACTIVE(I->ctl)) return;  // stopped, or out of iterations
     const int ti = __ldg(a.first + ii) + (g - __ldg(a.prefix + ii));
@@ -381,7 +394,7 @@ __device__ __forceinline__ void wide_tile(const SweepArgs& a, int g, int g_next,
     constexpr bool update = MODE == kFwdUpdate || MODE == kBwdUpdate;
     constexpr bool asc = MODE != kBwdUpdate;  // labels SP(., TOP) first, then the layers in ascending order
     prefetch_tile(a, g_next, lane);
-    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const int ii = find_inst_warp(a.prefix, a.n_inst, g, lane);
     const InstDev* __restrict__ I = a.insts + ii;
     if (update && FDOG_INACTIVE(I->ctl)) return;
     const int ti = __ldg(a.first + ii) + (g - __ldg(a.prefix + ii));
@@ -627,7 +640,7 @@ __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, 
     float* ep_lam = wsm + static_cast<size_t>(a.kstride) * W * kTile;
     int* ep_var = reinterpret_cast<int*>(ep_lam + static_cast<size_t>(a.epi) * kTile);
     prefetch_tile(a, g_next, lane);
-    const int ii = find_inst(a.prefix, a.n_inst, g);
+    const int ii = find_inst_warp(a.prefix, a.n_inst, g, lane);
     const InstDev* __restrict__ I = a.insts + ii;
     if (update && FDOG_INACTIVE(I->ctl)) return;
     const int ti = __ldg(a.first + ii) + (g - __ldg(a.prefix + ii));
