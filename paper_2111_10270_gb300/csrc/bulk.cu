@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <new>
 #include <vector>
 
 #include "instance.h"
@@ -14,12 +15,13 @@ namespace {
 
 constexpr int kBulkWarps = 8;
 constexpr int kBulkStages = 2;
-// The rule for bulk sweeps: at least this many tiles, so that the warps of a resident grid (some 4,900) have several
-// each to copy ahead, and three quarters of them plain.  200 iterations on grids, ms, ordinary and bulk sweeps: 4
-// labels, 18 k tiles 7.25 and 6.40, 34 k 9.95 and 8.58, 48 k 12.5 and 10.4; 2 labels (shorter rows), 33 k 8.23 and
-// 8.11, 66 k 13.2 and 12.1.  With 3 labels the edges that a tile's end cuts make every tile a mixed one, whose slots
-// all need ids and whose layers take both ways: 31 k tiles 14.8 and 16.3.  Below, with 9.6 k tiles, 15.5 and 16.2.
-constexpr int32_t kBulkMinTiles = 16384;
+// The rule for bulk sweeps: three quarters of the tiles plain, and at least this many of them.  200 iterations on grids,
+// ms, ordinary and bulk sweeps: 4 labels, 0.28 k tiles 3.43 and 3.40, 2.1 k 4.31 and 3.91, 8.7 k 5.37 and 5.10, 18 k 7.25
+// and 6.40, 48 k 12.5 and 10.4; 8 labels, 0.56 k tiles 3.90 and 3.72, 4.2 k 5.97 and 4.82.  Rows of three layers
+// (2 labels) leave little to form from a copied tile: 4.2 k tiles 4.08 and 4.33, 10 k 5.05 and 5.13, 33 k 8.23 and 8.11,
+// 66 k 13.2 and 12.1.  With 3 labels the edges that a tile's end cuts make every tile a mixed one, whose slots all need
+// ids and whose layers take both ways: 31 k tiles 14.8 and 16.3.
+constexpr int32_t kBulkMinTiles = 256, kBulkMinShortTiles = 16384;
 constexpr int64_t kBulkMaxPatterns = 64;  // a tile's table entry has 8 bits for its pattern; more would be large tables
 
 size_t smem_of(int stages, int rows) {
@@ -59,15 +61,20 @@ __global__ void __launch_bounds__(256) bulk_targets_kernel(const InstDev* insts,
 
 bool bulk_possible(const Decomposition& d) {
     const int64_t np = static_cast<int64_t>(d.patterns.size() / 2);
-    if (np < 1 || np > kBulkMaxPatterns || !d.cls_has_local[kJitClass] ||
-        d.cls_tile_begin[kJitClass + 1] - d.cls_tile_begin[kJitClass] < kBulkMinTiles)
-        return false;
+    const int32_t t0 = d.cls_tile_begin[kJitClass], n = d.cls_tile_begin[kJitClass + 1] - t0;
+    if (np < 1 || np > kBulkMaxPatterns || !d.cls_has_local[kJitClass] || n < kBulkMinTiles) return false;
+    if (n < kBulkMinShortTiles) {
+        int64_t layers = 0;
+        for (int32_t t = 0; t < n; ++t) layers += d.shapes[d.tiles[t0 + t].shape].k;
+        if (2 * layers < 9 * static_cast<int64_t>(n)) return false;  // fewer than 4.5 a row
+    }
     int shapes = 0;
     for (int c : d.shape_cls) shapes += c == kJitClass;
     return shapes <= FDOG_BULK_RUNS;
 }
 
-void plan_bulk(Decomposition& d, const uint16_t* local_ent) {
+// Without memory for it the instance runs the ordinary sweeps.
+void plan_bulk(Decomposition& d, const uint16_t* local_ent) try {
     d.bulk_runs.clear();
     d.bulk_pairs.clear();
     const size_t np = d.patterns.size() / 2;
@@ -153,6 +160,8 @@ void plan_bulk(Decomposition& d, const uint16_t* local_ent) {
     d.bulk_rows = rows;
     d.bulk_cv_rows = row;
     d.bulk_pairs = std::move(pairs);
+} catch (const std::bad_alloc&) {
+    d.bulk_runs.clear();
 }
 
 int setup_bulk(fdog_instance* inst) {

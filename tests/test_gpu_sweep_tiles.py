@@ -151,8 +151,10 @@ def join(*parts):
 
 # Instances that run bulk sweeps: grids whose edges fill their tiles (4, 2 and 8 labels), and one of them beside
 # grids whose edges are cut by the tile's end (slots of one layer of both kinds), rows of variables with one copy,
-# partial last tiles and tiles without any local variable.
+# partial last tiles and tiles without any local variable; then the smallest, with fewer tiles than resident warps.
 BULK = {
+    "4 small": lambda: ilpgen.mrf_grid(23, 24, 4, 3, potts_max=2.0),
+    "8 small": lambda: ilpgen.mrf_grid(17, 19, 8, 3, potts_max=2.0),
     "4": lambda: ilpgen.mrf_grid(190, 190, 4, 3, potts_max=2.0),
     "2": lambda: ilpgen.mrf_grid(370, 361, 2, 3, potts_max=2.0),
     "8": lambda: ilpgen.mrf_grid(131, 133, 8, 3, potts_max=2.0),
