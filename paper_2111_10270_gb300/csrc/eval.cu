@@ -48,8 +48,16 @@ __device__ __forceinline__ double pick64(const double (&x)[W], uint32_t code) {
 // E^j of the BDD in `lane` of a tile: SP(root, TOP) with arcs leaving layer t
 // costing lambda_t on the 1-arc and 0 on the 0-arc (Def. 4, Fig. 3).  With
 // add_t the multiplier of a slot is first formed as the FP32 sum lambda + T,
-// exactly as the add-back (Alg. 1, last loop) stores it.
-template <int W>
+// exactly as the add-back (Alg. 1, last loop) stores it.  STRIDE: codes of a
+// layer in the template, of which the first W are its nodes'.
+//
+// FP64 additions and minima run at two per clock and SM here, so they are what
+// bounds this: a template of four nodes per layer took eight of them a slot
+// (258 us for 5.5 M slots of width-2 BDDs, 224 as below).  Width-2 rows in such a template
+// are walked as width 2, and their inner layers, one of two structures (see
+// kStepUp), take one addition and one minimum: the other node's label is its
+// successor's.  The same minima of the same sums.
+template <int W, int STRIDE>
 __device__ double bdd_energy64(const InstDev* __restrict__ I, const TileDev& tile, const ShapeDev& sh, int lane,
                                bool add_t) {
     const uint16_t* __restrict__ tpl = I->tpl + sh.tpl_off;
@@ -57,20 +65,35 @@ __device__ double bdd_energy64(const InstDev* __restrict__ I, const TileDev& til
     double nx[W];
 #pragma unroll
     for (int v = 0; v < W; ++v) nx[v] = dinf();
+#pragma unroll 4
     for (int t = sh.k - 1; t >= 0; --t) {
         const size_t p = base + static_cast<size_t>(t) * kTile;
         float l = I->lam[p];
         if (add_t) l += I->T[I->var[p]];
         const double lt = static_cast<double>(l);
         uint32_t c[W];
-        load_codes<W>(tpl + t * W, c);
-        double cur[W];
+        load_codes<W>(tpl + t * STRIDE, c);
+        if (W == 2 && (c[0] | c[1] << 16) == dev::kStepUp) {
+            nx[0] = fmin(nx[0], nx[1] + lt);
+        } else if (W == 2 && (c[0] | c[1] << 16) == dev::kStepDown) {
+            nx[1] = fmin(nx[1], nx[0] + lt);
+        } else {
+            double cur[W];
 #pragma unroll
-        for (int v = 0; v < W; ++v) cur[v] = fmin(pick64<W>(nx, c[v] & 0xFFu), pick64<W>(nx, c[v] >> 8) + lt);
+            for (int v = 0; v < W; ++v) cur[v] = fmin(pick64<W>(nx, c[v] & 0xFFu), pick64<W>(nx, c[v] >> 8) + lt);
 #pragma unroll
-        for (int v = 0; v < W; ++v) nx[v] = cur[v];
+            for (int v = 0; v < W; ++v) nx[v] = cur[v];
+        }
     }
     return nx[0];
+}
+
+// whether the layers of a four-node template have at most two nodes (all lanes call it)
+__device__ __forceinline__ bool narrow_in_4(const uint16_t* __restrict__ tpl, int k, int lane) {
+    bool two = true;
+    for (int t = lane; t < k; t += kTile)
+        two = two && __ldg(reinterpret_cast<const unsigned int*>(tpl + t * 4) + 1) == 0xFFFFFFFFu;
+    return __all_sync(0xffffffffu, two);
 }
 
 struct Eval64Args {
@@ -94,15 +117,15 @@ __global__ void __launch_bounds__(256) eval64_kernel(Eval64Args a) {
     double s = 0.0, cp = 0.0;
     for (int ti = c * kLbChunk + wib; ti < t_end; ti += 8) {
         const TileDev tile = I->tiles[ti];
-        if (lane >= tile.n_valid) continue;
         const ShapeDev sh = I->shapes[tile.shape];
+        const bool two = sh.width == 2 || (sh.width == 4 && narrow_in_4(I->tpl + sh.tpl_off, sh.k, lane));
+        if (lane >= tile.n_valid) continue;
+        const bool add_t = a.add_t != 0;
         double e;
-        switch (sh.width) {
-            case 2: e = bdd_energy64<2>(I, tile, sh, lane, a.add_t != 0); break;
-            case 4: e = bdd_energy64<4>(I, tile, sh, lane, a.add_t != 0); break;
-            case 8: e = bdd_energy64<8>(I, tile, sh, lane, a.add_t != 0); break;
-            default: e = bdd_energy64<16>(I, tile, sh, lane, a.add_t != 0); break;
-        }
+        if (two) e = sh.width == 2 ? bdd_energy64<2, 2>(I, tile, sh, lane, add_t) : bdd_energy64<2, 4>(I, tile, sh, lane, add_t);
+        else if (sh.width == 4) e = bdd_energy64<4, 4>(I, tile, sh, lane, add_t);
+        else if (sh.width == 8) e = bdd_energy64<8, 8>(I, tile, sh, lane, add_t);
+        else e = bdd_energy64<16, 16>(I, tile, sh, lane, add_t);
         neumaier64(s, cp, e);
     }
     // fixed-order block reduction: butterfly per warp, then warp 0 over the 8 warp totals

@@ -213,3 +213,23 @@ def test_bulk_sweeps_match_the_ordinary_ones(P, name):
     assert a.iterate(4) == b.iterate(4)
     assert a.primal_round() == b.primal_round()
     same()
+
+
+@pytest.mark.parametrize("add_back", [False, True])
+@pytest.mark.parametrize("name", ["amo2", "amo8", "amo9", "flow16", "product", "marg6", "cover7", "card6", "exact5",
+                                  "mixed12"])
+def test_evaluation_of_specialised_rows(P, oracle_mod, name, add_back):
+    """Rows of width 2 beside wider ones, most in templates of four nodes per layer: the evaluated bound is the
+    oracle's."""
+    g = join(rows_ilp(*PATTERNS[name], 33, 5, True), rows_ilp(*PATTERNS["card6"], 31, 6, False))
+    inst = P.Instance.from_ilp(g, P.capi.default_params(tol=0.0, jit=1)).build(0)
+    orc = oracle_mod.Problem.from_ilp(g)
+    assert inst.kernel_plan()["jit_tiles"] > 0
+    for _ in range(4):
+        inst.iterate(1)
+        orc.iterate(1)
+    if add_back:
+        inst.finalize()
+        orc.addback()
+    _, fea = inst.lower_bound()
+    assert lb_close(fea, orc.lower_bounds()[1], scale=np.abs(orc.energies()).sum())
