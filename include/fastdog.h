@@ -567,14 +567,14 @@ int fdog_shard_commit(fdog_instance* inst, double lb, int32_t* stop);
  * serves callers that cannot allocate device memory -- plug-ins whose host
  * framework owns every device allocation through its own pool, and real-time
  * loops that forbid allocation after start-up).
- * Writes to dev_out[0] the deterministic FP64 compensated sum
+ * Writes to dev_out[0] the deterministic sum
  * constant + sum_{t < n} dev_values[t] -- e.g. per-subproblem energies E_j, so
- * that the result is the bound sum_j E^j of Eq. D -- with the same two-stage
- * compensated reduction as the library's own bound kernels: per-block
- * partials (256 values per block), then a last-block Neumaier sum of them.
+ * that the result is the bound sum_j E^j of Eq. D: the values are added as
+ * 128-bit fixed-point numbers, per block and then by the last block, and the
+ * total is rounded once.
  * dev_values (n doubles) and dev_out (one double) are device memory owned by
  * the caller; the call allocates nothing: its scratch is a static device
- * array of 256 KiB that every GPU loading this library holds until the
+ * array of about 32 KiB that every GPU loading this library holds until the
  * process exits.  n = 0 writes `constant`.
  * n may be at most 8,388,608 (FDOG_EINVAL beyond, or for negative n or NULL
  * pointers).  The first call on a device looks up that array's device address

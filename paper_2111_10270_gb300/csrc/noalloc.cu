@@ -14,12 +14,13 @@
 // the read of the values: FP64 additions run at two per clock and SM on this
 // part, so that the compensated FP64 tree over 256 values per block that
 // stood here took 142 us for 4,000,037 values; integer shifts and additions
-// run at the full rate (18.5 us).  Scratch -- the block totals and the last-block ticket
-// -- is one file-scope static device array instead of memory owned by an
+// run at the full rate (18.5 us).  Scratch -- the block totals and the last-block
+// tickets -- is one file-scope static device array instead of memory owned by an
 // instance.
 #include <cuda.h>  // CUcontext / CUresult types of the two driver calls fetched at run time
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <mutex>
 
@@ -36,10 +37,13 @@ constexpr int64_t kMaxValues = int64_t(1) << 23;  // 8,388,608 values per call
 constexpr int kMaxBlocks = static_cast<int>(kMaxValues / (kThreads * kManyPer));
 static_assert(kFewMax / (kThreads * kFewPer) <= kMaxBlocks, "scratch holds the totals of either kind");
 constexpr int kMaxDevices = 64;
+constexpr unsigned kTickets = 64;
 
 struct Scratch {
     double part[2 * kMaxBlocks];  // total of each block: leading part, remainder
-    unsigned ticket;              // wraps to zero with the last block of a call
+    // A call's last-block ticket, which wraps to zero with its last block.  Calls take them in turn, so that calls
+    // that overlapped, with wrong sums in `part`, leave every ticket at zero all the same, and no memset is needed.
+    unsigned ticket[kTickets];
 };
 
 // Held by every GPU that loads this library until the process exits.  In host
@@ -51,6 +55,7 @@ std::mutex g_mu;
 // per device: the scratch address and the id of the context it was looked up in
 Scratch* g_addr[kMaxDevices] = {};
 unsigned long long g_ctx[kMaxDevices] = {};
+std::atomic<unsigned> g_calls{0};
 
 // Fixed-point sums.  A value of biased exponent e (1 for subnormal numbers) is
 // m 2^(e - 1075) with a 53-bit m; beside values of largest exponent emax it is
@@ -137,7 +142,7 @@ __device__ __forceinline__ double2 to_pair(Fixed a, int emax) {
 template <int PER>
 __global__ void __launch_bounds__(kThreads) bound_reduce_noalloc_kernel(const double* __restrict__ v, int64_t n,
                                                                          double constant, double* __restrict__ out,
-                                                                         Scratch* scr) {
+                                                                         Scratch* scr, unsigned call) {
     __shared__ bool last;
     const int64_t first = static_cast<int64_t>(blockIdx.x) * (kThreads * PER) + threadIdx.x;
     double x[PER];
@@ -156,7 +161,7 @@ __global__ void __launch_bounds__(kThreads) bound_reduce_noalloc_kernel(const do
         scr->part[2 * blockIdx.x] = p.x;
         scr->part[2 * blockIdx.x + 1] = p.y;
         __threadfence();
-        last = atomicInc(&scr->ticket, gridDim.x - 1) == gridDim.x - 1;
+        last = atomicInc(scr->ticket + call % kTickets, gridDim.x - 1) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
@@ -251,8 +256,9 @@ extern "C" int fdog_bound_reduce_noalloc(const double* dev_values, int64_t n, do
     const bool few = n <= kFewMax;
     const int64_t per_block = kThreads * (few ? kFewPer : kManyPer);
     const unsigned blocks = n > 0 ? static_cast<unsigned>((n + per_block - 1) / per_block) : 1u;
-    if (few) bound_reduce_noalloc_kernel<kFewPer><<<blocks, kThreads, 0, s>>>(dev_values, n, constant, dev_out, scr);
-    else bound_reduce_noalloc_kernel<kManyPer><<<blocks, kThreads, 0, s>>>(dev_values, n, constant, dev_out, scr);
+    const unsigned call = g_calls.fetch_add(1, std::memory_order_relaxed);
+    if (few) bound_reduce_noalloc_kernel<kFewPer><<<blocks, kThreads, 0, s>>>(dev_values, n, constant, dev_out, scr, call);
+    else bound_reduce_noalloc_kernel<kManyPer><<<blocks, kThreads, 0, s>>>(dev_values, n, constant, dev_out, scr, call);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? FDOG_OK : FDOG_ECUDA;
 }
