@@ -58,7 +58,7 @@ METRIC = ("BDD arc-updates/s (full FastDOG solve: dual iterations up to the work
           "stopping early at the 1e-4 LB-gap rule, + perturbation rounding)")
 UNIT = "arc-updates/s"
 SWEEP_SRCS = [os.path.join(ROOT, "paper_2111_10270_gb300", "csrc", f)
-              for f in ("jit.cpp", "jit_skeleton.cuh", "kernels.cu")]  # generator, skeleton, launch (L2 window)
+              for f in ("jit.cpp", "jit_skeleton.cuh", "bulk.cu", "kernels.cu")]  # generator, skeleton, plan, launch (L2 window)
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "sweep_traffic.txt")
 
 
@@ -537,7 +537,7 @@ def iteration_bytes(kp, info):
     deferred-sum passes): every array element counted once per launch (see
     the roofline block of main)."""
     tiles = kp["jit_tiles"] + kp["static_tiles"]
-    sweep = 12 * info["n_slots"] + 4 * (kp["local_vars"] + kp["work_vars"]) + 40 * tiles + 8 * kp["local_vars"]
+    sweep = 12 * info["n_slots"] + 4 * kp["work_vars"] + 40 * tiles
     reduce = 12 * kp["work_vars"] + 8 * kp["work_slots"]
     return sweep, reduce, 2 * (sweep + reduce)
 
@@ -738,15 +738,15 @@ def main():
 
     # ---- roofline of the dominant kernel (update sweep) ----------------------
     kp = inst.kernel_plan()
-    S = info["n_slots"]
     n_bdds = info["n_bdds"]
     tiles = kp["jit_tiles"] + kp["static_tiles"]
-    n_row_vars = kp["local_vars"] + kp["work_vars"]  # variables inside some BDD
-    # compulsory bytes of one sweep launch, every array element counted once: per slot lambda read + write
-    # and its variable id (12 B); per variable in a row its deferred term T, read once (4 B; the per-slot
-    # gathers of T beyond the first are re-reads the L2 serves); per tile its descriptor and bound partial
-    # (40 B); per tile-local variable its target C and new deferred term (8 B)
-    alg_bytes = 12 * S + 4 * n_row_vars + 40 * tiles + 8 * kp["local_vars"]
+    # compulsory bytes of one sweep launch, every array element counted once: per slot lambda read + write and one
+    # more word, the id of a variable with copies in several tiles or the target C of a tile-local one, whose
+    # deferred term the bulk sweeps form from the tile's multipliers (12 B); per variable with copies in several
+    # tiles its deferred term T, read once (4 B; the gathers beyond the first are re-reads the L2 serves); per tile
+    # its descriptor and bound partial (40 B).  The sweeps that store and read the tile-local terms move 12 B more
+    # per tile-local variable; they are measured against the same bytes.
+    alg_bytes = iteration_bytes(kp, info)[0]
     # per deferred-sum launch: per listed variable its id, C and the new T (12 B); per copy its slot
     # position and the gathered multiplier (8 B)
     reduce_bytes = 12 * kp["work_vars"] + 8 * kp["work_slots"]
@@ -757,7 +757,8 @@ def main():
     peak_src = "measured" if peak else "fallback"
     if not peak:
         peak = 6800.0
-    kernel_name = ("fdog_jit_fwd / fdog_jit_bwd (shape-specialised update sweeps)" if kp["jit_tiles"] * 2 >= tiles
+    kernel_name = ("shape-specialised update sweeps (fdog_bulk_fwd / _bwd on regular instances, else fdog_jit_fwd / _bwd)"
+                   if kp["jit_tiles"] * 2 >= tiles
                    else "update sweeps of the dominant kernel class")
     traffic = sweep_traffic(args.workload)
     dram_gbs = traffic / sweep_avg_s / 1e9 if (traffic and sweep_avg_s > 0) else None
@@ -854,7 +855,7 @@ def main():
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": elapsed / args.steps * 1e3, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
-            "config": {"workload": w["desc"], "vars": info["n_vars"], "bdds": n_bdds, "slots": S, "nodes": nodes,
+            "config": {"workload": w["desc"], "vars": info["n_vars"], "bdds": n_bdds, "slots": info["n_slots"], "nodes": nodes,
                        "dual_iters_per_step": dual_iters / args.steps, "stop_iters": last["iters"],
                        "rounds": last["rounds"], "rounding_status": last["rc"], "lb": last["lb"], "ub": last["obj"],
                        "feasible": last["feasible"],
