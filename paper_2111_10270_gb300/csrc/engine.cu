@@ -576,10 +576,16 @@ int view_autotune(Engine& e, BatchView& v, bool tune_grid) {
     // iterations per graph replay: about 1 ms of device work per replay (an
     // iteration costs about two and a half sweeps; four sweeps were timed), so
     // that the status read after a replay stays a small fraction of it;
-    // results do not depend on it
+    // results do not depend on it.  With several members four: each of them
+    // runs its own rounding rounds of some twenty iterations, and a round and
+    // a stop wait for the end of a replay with the others' work going on
+    // (batches of 12, 8 and 4 cell-tracking instances, ms: 95.5, 55.1 and
+    // 31.8 as for one instance, 86.7, 50.3 and 30.7 with at most eight, 83.7,
+    // 49.3 and 29.8 with four)
     const double iter_ms = 2.5 * best_ms / 4.0;
+    const int most = v.members.size() > 1 ? 4 : 32;
     int chunk = 4;
-    while (chunk < 32 && chunk * iter_ms < 1.0) chunk *= 2;
+    while (chunk < most && chunk * iter_ms < 1.0) chunk *= 2;
     e.chunk = chunk;
     return FDOG_OK;
 }
