@@ -570,8 +570,10 @@ int fdog_shard_commit(fdog_instance* inst, double lb, int32_t* stop);
  * Writes to dev_out[0] the deterministic sum
  * constant + sum_{t < n} dev_values[t] -- e.g. per-subproblem energies E_j, so
  * that the result is the bound sum_j E^j of Eq. D: the values are added as
- * 128-bit fixed-point numbers, per block and then by the last block, and the
- * total is rounded once.
+ * integers over the whole range of FP64, so that the sum is exact whatever
+ * their order and size, and is rounded at the end; *dev_out is within one unit
+ * in the last place of the exact sum, or NaN if a value or the constant is not
+ * finite or the total is beyond the largest double.
  * dev_values (n doubles) and dev_out (one double) are device memory owned by
  * the caller; the call allocates nothing: its scratch is a static device
  * array of about 32 KiB that every GPU loading this library holds until the
