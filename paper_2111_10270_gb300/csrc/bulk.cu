@@ -182,8 +182,7 @@ int setup_bulk(fdog_instance* inst) {
     int most = 1 << 30;
     for (int m = 0; m < 2; ++m) {
         int n = 0;
-        if (cudaFuncSetAttribute(inst->jit.bulk[m], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem)) != cudaSuccess ||
+        if (allow_smem(inst->jit.bulk[m], smem) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, inst->jit.bulk[m], 32 * kBulkWarps, smem) != cudaSuccess) {
             cudaGetLastError();
             n = 0;
@@ -200,7 +199,7 @@ cudaError_t launch_bulk(const DevBatch& b, int mode, const LaunchCfg& cfg, cudaS
     args.inst = b.insts;
     const size_t smem = smem_of(args.stages, args.rows);
     const void* fn = b.jit.bulk[mode];
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     const int blocks = std::min(b.bulk.blocks_per_sm * cfg.num_sms, (args.total + kBulkWarps - 1) / kBulkWarps);
     void* kargs[] = {&args};

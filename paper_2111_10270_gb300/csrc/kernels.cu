@@ -19,6 +19,10 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <map>
+#include <mutex>
+#include <new>
+#include <utility>
 
 #include "kernels.h"
 #include "reduce.cuh"
@@ -506,10 +510,7 @@ cudaError_t launch_class(const DevBatch& b, int cls, int mode, int mm_flags, con
         e = launch_bulk(b, mode, cfg, s);
     } else if (cls == kJitClass) {
         void* kargs[] = {&args};
-        e = cudaSuccess;
-        if (smem > 48 * 1024)
-            e = cudaFuncSetAttribute(b.jit.fn[mode], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem));
+        e = allow_smem(b.jit.fn[mode], smem);
         if (e == cudaSuccess) e = launch_windowed(b.jit.fn[mode], blocks, 32 * wpb, kargs, smem, s, l2);
     } else switch (W) {
         case 2: e = launch_sweep_width<2>(reg, mode, blocks, 32 * wpb, smem, s, args, l2); break;
@@ -526,6 +527,24 @@ cudaError_t launch_class(const DevBatch& b, int cls, int mode, int mm_flags, con
 bool can_fork(const LaunchCfg& cfg) { return cfg.side && cfg.side->ready; }
 
 }  // namespace
+
+cudaError_t allow_smem(const void* fn, size_t bytes) try {
+    if (bytes <= 48 * 1024) return cudaSuccess;  // every kernel's limit to begin with
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> limits;  // per device and kernel
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    size_t& limit = limits[{dev, fn}];
+    const size_t most = std::max(limit, bytes);
+    // set again each time: a device that was reset has forgotten it
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+    if (e == cudaSuccess) limit = most;
+    return e;
+} catch (const std::bad_alloc&) {
+    return cudaErrorMemoryAllocation;
+}
 
 cudaError_t launch_windowed(const void* fn, int blocks, int threads, void** args, size_t smem, cudaStream_t s,
                             const L2Window& l2) {

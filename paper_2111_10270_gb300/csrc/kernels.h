@@ -54,6 +54,11 @@ struct L2Window {
 // device maximum; never lowered) and returns the window for [base, base + bytes).
 L2Window l2_window_for(int device, void* base, size_t bytes);
 
+// Lets `fn` be launched with `bytes` of dynamic shared memory on the current
+// device.  The limit belongs to the kernel, which instances on other host
+// threads may be launching or capturing with more, so it is never lowered.
+cudaError_t allow_smem(const void* fn, size_t bytes);
+
 // a kernel launch with programmatic stream serialization (the kernel calls
 // pdl_wait before it touches memory) and an optional L2 access-policy window
 // (kernels.cu)

@@ -189,12 +189,8 @@ cudaError_t launch_persistent(const DevBatch& b, int iters, unsigned* bar, doubl
     a.bar = bar;
     a.wait_ns = static_cast<unsigned long long>(std::max(wait_s, 0.0) * 1e9);
     int per_sm = 0;
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(persist_iterations_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(persist_iterations_kernel), smem);
+    if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persist_iterations_kernel, kPersistThreads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;

@@ -875,11 +875,8 @@ inline auto seg_fn(int mode) -> void (*)(SweepArgs) {
         void (*fn)(SweepArgs);                                                                                 \
         if constexpr (W <= kRegW) fn = reg ? dev::sweep_fn<W, true>(mode) : dev::seg_fn<W>(mode);              \
         else fn = dev::sweep_fn<W, false>(mode);                                                               \
-        if (smem > 48 * 1024) {                                                                                \
-            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,              \
-                                                 static_cast<int>(smem));                                      \
-            if (e != cudaSuccess) return e;                                                                    \
-        }                                                                                                      \
+        const cudaError_t e = allow_smem(reinterpret_cast<const void*>(fn), smem);                             \
+        if (e != cudaSuccess) return e;                                                                        \
         void* args[] = {const_cast<SweepArgs*>(&a)};                                                           \
         return launch_windowed(reinterpret_cast<const void*>(fn), blocks, threads, args, smem, s, l2);         \
     }

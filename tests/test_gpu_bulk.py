@@ -1,0 +1,54 @@
+"""GPU tests of the bulk sweeps' plan and of what instances that run them share."""
+import threading
+
+import pytest
+
+import ilpgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2111_10270_gb300 import build as b
+
+    b.build()
+    import paper_2111_10270_gb300 as fdog
+
+    return fdog
+
+
+def grid(P, h, w, labels, **kw):
+    ilp = ilpgen.mrf_grid(h, w, labels, 3, potts_max=2.0)
+    return P.Instance.from_ilp(ilp, P.capi.default_params(tol=0.0, jit=1, **kw))
+
+
+def test_instances_of_common_kernels_on_two_threads(P):
+    """Both run the kernels of the same shapes with shared memory of their own size; profiling launches every pass by
+    itself, outside of graphs."""
+    import torch
+
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    insts = [grid(P, h, w, 4).build(0, s) for (h, w), s in zip([(190, 190), (100, 101)], streams)]
+    want = [(i.iterate(800), i.reset())[0] for i in insts]
+    errors, got = [], [None, None]
+
+    def work(q):
+        try:
+            for _ in range(200):
+                got[q] = insts[q].iterate(4)
+        except Exception as e:
+            errors.append(repr(e))
+
+    for i in insts:
+        i.set_profiling(True)
+    threads = [threading.Thread(target=work, args=(q,)) for q in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert errors == []
+    assert [g[1] for g in got] == [w[1] for w in want]
