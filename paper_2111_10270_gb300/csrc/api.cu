@@ -8,6 +8,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "engine.h"
@@ -144,6 +145,38 @@ static int check_layer_limits(fdog_instance* inst) {
     return FDOG_OK;
 }
 
+// Compiles the modules of a planned instance's shapes, that of its bulk sweeps beside the other.  Without the former
+// it runs the ordinary sweeps.
+static int compile_modules(fdog_instance* inst, std::string& why) {
+    const std::vector<int> ids = jit_ids(inst), bulk = bulk_ids(inst);
+    int bulk_rc = FDOG_OK;
+    auto compile_bulk = [&] {
+        try {
+            std::string unused;
+            bulk_rc = jit_compile(bulk, unused, true);
+        } catch (...) {
+            bulk_rc = FDOG_ENOMEM;
+        }
+    };
+    std::thread beside;
+    if (!jit_compiled(bulk, true)) {
+        try {
+            beside = std::thread(compile_bulk);
+        } catch (...) {
+            compile_bulk();
+        }
+    }
+    int rc = FDOG_OK;
+    try {
+        rc = jit_compile(ids, why);
+    } catch (...) {
+        rc = FDOG_ENOMEM;
+    }
+    if (beside.joinable()) beside.join();
+    if (bulk_rc != FDOG_OK) inst->dec.bulk_runs.clear();
+    return rc;
+}
+
 int plan(fdog_instance* inst, bool compile_jit) {
     if (inst->planned) return FDOG_OK;
     free_device_plan(inst->dec, inst->stream);
@@ -166,10 +199,9 @@ int plan(fdog_instance* inst, bool compile_jit) {
     if ((rc = check_layer_limits(inst)) != FDOG_OK) return rc;
     if (inst->params.update == 1) build_serial_schedule(inst->n_vars, inst->dec);
     if (bulk_wanted(inst) && bulk_possible(inst->dec)) plan_bulk(inst->dec, inst->dec.local_ent.data());
-    std::vector<int> ids = jit_ids(inst);
-    if (compile_jit && !ids.empty()) {
+    if (compile_jit && !jit_ids(inst).empty()) {
         std::string why;
-        if (jit_compile(ids, why) != FDOG_OK) {
+        if (compile_modules(inst, why) != FDOG_OK) {
             // shape-specialised kernels unavailable: plan again for the generic kernels only
             inst->jit_note = why;
             inst->jit_failed = true;
@@ -193,9 +225,8 @@ static int plan_for_build(fdog_instance* inst) {
                 free_device_plan(inst->dec, inst->stream);
                 return rc;
             }
-            std::vector<int> ids = jit_ids(inst);
             std::string why;
-            if (!ids.empty() && jit_compile(ids, why) != FDOG_OK) {
+            if (!jit_ids(inst).empty() && compile_modules(inst, why) != FDOG_OK) {
                 inst->jit_note = why;
                 inst->jit_failed = true;
                 free_device_plan(inst->dec, inst->stream);
@@ -600,6 +631,9 @@ int build_instance(fdog_instance* inst, int32_t device, void* cuda_stream, bool 
             if ((rc = plan_for_build(inst)) != FDOG_OK) return rc;
         }
     }
+    const std::vector<int> bulk = bulk_ids(inst);
+    std::string unused;
+    if (!bulk.empty() && jit_kernels(bulk, inst->bulk_jit, unused, true) != FDOG_OK) inst->dec.bulk_runs.clear();
     cudaDeviceProp prop;
     e = cudaGetDeviceProperties(&prop, device);
     if (e != cudaSuccess) return fail_cuda(inst, e, "device properties");

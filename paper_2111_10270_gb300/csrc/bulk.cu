@@ -164,11 +164,18 @@ void plan_bulk(Decomposition& d, const uint16_t* local_ent) try {
     d.bulk_runs.clear();
 }
 
+std::vector<int> bulk_ids(const fdog_instance* inst) {
+    std::vector<int> ids;
+    if (bulk_wanted(inst))
+        for (const BulkRun& r : inst->dec.bulk_runs) ids.push_back(r.jit);
+    return ids;
+}
+
 int setup_bulk(fdog_instance* inst) {
     BulkPlan& plan = inst->batch.bulk;
     plan = BulkPlan();
     const Decomposition& d = inst->dec;
-    if (!inst->hdesc.cv || !inst->jit.bulk[0]) return FDOG_OK;
+    if (!inst->hdesc.cv) return FDOG_OK;
     const DevArrays& a = inst->dev;
     cudaError_t e = copy_async(inst, a.bulk_runs, d.bulk_runs.data(), sizeof(BulkRun) * d.bulk_runs.size(),
                                cudaMemcpyHostToDevice);
@@ -182,8 +189,9 @@ int setup_bulk(fdog_instance* inst) {
     int most = 1 << 30;
     for (int m = 0; m < 2; ++m) {
         int n = 0;
-        if (allow_smem(inst->jit.bulk[m], smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, inst->jit.bulk[m], 32 * kBulkWarps, smem) != cudaSuccess) {
+        plan.fn[m] = inst->bulk_jit.fn[m];
+        if (allow_smem(plan.fn[m], smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, plan.fn[m], 32 * kBulkWarps, smem) != cudaSuccess) {
             cudaGetLastError();
             n = 0;
         }
@@ -198,7 +206,7 @@ cudaError_t launch_bulk(const DevBatch& b, int mode, const LaunchCfg& cfg, cudaS
     BulkArgs args = b.bulk.args;
     args.inst = b.insts;
     const size_t smem = smem_of(args.stages, args.rows);
-    const void* fn = b.jit.bulk[mode];
+    const void* fn = b.bulk.fn[mode];
     const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     const int blocks = std::min(b.bulk.blocks_per_sm * cfg.num_sms, (args.total + kBulkWarps - 1) / kBulkWarps);

@@ -398,15 +398,18 @@ void build_serial_schedule(int32_t n_vars, Decomposition& d);
 // shape-specialised code (jit.cpp): process-wide shape registry and kernels
 int jit_register_shape(const HostShape& s);  // id of the shape's structure
 struct JitKernels {
-    const void* fn[4] = {nullptr, nullptr, nullptr, nullptr};  // per sweep mode
-    const void* bulk[2] = {nullptr, nullptr};                  // bulk sweeps: ascending, descending pass
+    const void* fn[4] = {nullptr, nullptr, nullptr, nullptr};  // per sweep mode; bulk sweeps: ascending, descending pass
 };
+// A set of shapes has a module of its sweeps and, where an instance runs them,
+// one of its bulk sweeps (bulk): these take as long to compile as the others.
 // host-only NVRTC compile of the module for the given shape ids (cached)
-int jit_compile(const std::vector<int>& ids, std::string& err);
+int jit_compile(const std::vector<int>& ids, std::string& err, bool bulk = false);
+// whether that would find the module compiled
+bool jit_compiled(const std::vector<int>& ids, bool bulk);
 // compiles if needed and loads the module; empty ids -> no kernels
-int jit_kernels(const std::vector<int>& ids, JitKernels& out, std::string& err);
+int jit_kernels(const std::vector<int>& ids, JitKernels& out, std::string& err, bool bulk = false);
 // the generated CUDA source of the module (for inspection)
-std::string jit_source(const std::vector<int>& ids);
+std::string jit_source(const std::vector<int>& ids, bool bulk = false);
 
 // The BDD of one row (coefficients of its non-zero entries in ascending
 // variable order, no variable fixed); `presolve` is set when the row forces

@@ -99,6 +99,7 @@ struct fdog_instance {
     bool solution_pinned = false;       // the last solution lives in host_x (else in `solution`)
     fdog::Profiler prof;
     fdog::JitKernels jit;     // shape-specialised kernels of this instance's shapes
+    fdog::JitKernels bulk_jit;  // and the bulk sweeps, if it runs them
     bool jit_failed = false;  // NVRTC unavailable or failed: generic kernels only
     std::string jit_note;
 
@@ -150,6 +151,7 @@ int addback(fdog_instance* inst);
 inline bool bulk_wanted(const fdog_instance* inst) {
     return !inst->bulk_off && inst->params.block_threads == 0 && inst->params.update == 0 && !inst->shard;
 }
+std::vector<int> bulk_ids(const fdog_instance* inst);  // shapes whose tiles run them
 int setup_bulk(fdog_instance* inst);
 // stores the tile-local terms that bulk sweeps of any of these instances (the members of b) left out of T
 cudaError_t flush_terms(const std::vector<fdog_instance*>& members, const DevBatch& b, const LaunchCfg& cfg,

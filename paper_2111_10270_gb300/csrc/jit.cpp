@@ -40,12 +40,12 @@ std::unordered_map<std::string, int> g_ids;
 std::vector<HostShape> g_shapes;
 std::map<std::string, JitKernels> g_modules;
 std::map<std::string, std::vector<char>> g_cubins;
-std::string generate_module(const std::vector<int>& ids);
+std::string generate_module(const std::vector<int>& ids, bool bulk);
 
-std::string id_key(std::vector<int>& ids) {
+std::string id_key(std::vector<int>& ids, bool bulk) {
     std::sort(ids.begin(), ids.end());
     ids.erase(std::unique(ids.begin(), ids.end()), ids.end());
-    std::string key;
+    std::string key = bulk ? "b" : "";
     for (int id : ids) key += std::to_string(id) + ",";
     return key;
 }
@@ -54,14 +54,14 @@ std::string id_key(std::vector<int>& ids) {
 // outside the registry lock, so threads planning different instances compile
 // in parallel; a thread that needs a module another thread is compiling waits
 // for it instead of compiling it again.
-int compile_module(const std::vector<int>& ids, const std::string& key, std::string& err) {
+int compile_module(const std::vector<int>& ids, const std::string& key, bool bulk, std::string& err) {
     std::string src;
     {
         std::unique_lock<std::mutex> lk(g_mu);
         g_cv.wait(lk, [&] { return !g_building.count(key); });
         if (g_cubins.count(key)) return FDOG_OK;
         g_building.insert(key);
-        src = generate_module(ids);
+        src = generate_module(ids, bulk);
     }
     std::vector<char> cubin;
     int rc = FDOG_OK;
@@ -271,37 +271,31 @@ void emit_shape(std::ostringstream& o, const HostShape& s, int id, int mode, boo
     o << "  return term;\n}\n\n";
 }
 
-std::string generate_module(const std::vector<int>& ids) {
+// Only the section of the skeleton whose dispatch is defined is compiled.
+std::string generate_module(const std::vector<int>& ids, bool bulk) {
     std::ostringstream o;
     o << "typedef int int32_t;\ntypedef unsigned int uint32_t;\ntypedef unsigned short uint16_t;\n"
          "typedef unsigned char uint8_t;\ntypedef long long int64_t;\ntypedef unsigned long long uint64_t;\n"
          "#define FDOG_INF __int_as_float(0x7f800000)\n";
     o << kJitAbi << "\n";
-    for (int id : ids)
-        for (int mode = 0; mode < 4; ++mode) emit_shape(o, g_shapes[id], id, mode);
+    const int modes = bulk ? 2 : 4;
     // multiplier at a byte offset of the tile; deferred term of a tile-local slot, as in fdog_tile_local_sums
-    o << "__device__ __forceinline__ float fdog_at(const float* sl, unsigned p) {\n"
+    if (bulk)
+        o << "__device__ __forceinline__ float fdog_at(const float* sl, unsigned p) {\n"
          "  return *(const float*)((const char*)sl + p);\n}\n"
          "__device__ __forceinline__ float fdog_pair_term(float C, float l, unsigned p, bool zero, const float* sl) {\n"
          "  float s = 0.f + l, inv = 1.f;\n"
          "  if (p != FDOG_PAIR_ONE) { s += fdog_at(sl, p); inv = 0.5f; }\n"
          "  return zero ? 0.f : (C - s) * inv;\n}\n\n";
     for (int id : ids)
-        for (int mode = 0; mode < 2; ++mode) emit_shape(o, g_shapes[id], id, mode, true);
-    o << "#define FDOG_DISPATCH(MODE) \\\n";
-    for (int mode = 0; mode < 4; ++mode) {
+        for (int mode = 0; mode < modes; ++mode) emit_shape(o, g_shapes[id], id, mode, bulk);
+    o << "#define " << (bulk ? "FDOG_BULK_DISPATCH" : "FDOG_DISPATCH") << "(MODE) \\\n";
+    for (int mode = 0; mode < modes; ++mode) {
         o << "  " << (mode ? "else " : "") << "if (MODE == " << mode << ") { switch (jit) { \\\n";
         for (int id : ids)
-            o << "    case " << id << ": term = shp_" << id << "_" << mode
-              << "(I, base, valid, a.flags, local, ep_lam + lane, ep_var + lane); break; \\\n";
-        o << "    default: break; } } \\\n";
-    }
-    o << "\n#define FDOG_BULK_DISPATCH(MODE) \\\n";
-    for (int mode = 0; mode < 2; ++mode) {
-        o << "  " << (mode ? "else " : "") << "if (MODE == " << mode << ") { switch (jit) { \\\n";
-        for (int id : ids)
-            o << "    case " << id << ": term = shb_" << id << "_" << mode
-              << "(lam, T, valid, omega, zero, plain, sl, sc, sv, pk, lane); break; \\\n";
+            o << "    case " << id << ": term = " << (bulk ? "shb_" : "shp_") << id << "_" << mode
+              << (bulk ? "(lam, T, valid, omega, zero, plain, sl, sc, sv, pk, lane)"
+                       : "(I, base, valid, a.flags, local, ep_lam + lane, ep_var + lane)") << "; break; \\\n";
         o << "    default: break; } } \\\n";
     }
     o << "\n" << kJitSkeleton;
@@ -321,24 +315,31 @@ int jit_register_shape(const HostShape& s) {
     return id;
 }
 
-int jit_compile(const std::vector<int>& ids_in, std::string& err) {
+int jit_compile(const std::vector<int>& ids_in, std::string& err, bool bulk) {
     if (ids_in.empty()) return FDOG_OK;
     std::vector<int> ids = ids_in;
-    const std::string key = id_key(ids);
-    return compile_module(ids, key, err);
+    const std::string key = id_key(ids, bulk);
+    return compile_module(ids, key, bulk, err);
 }
 
-int jit_kernels(const std::vector<int>& ids_in, JitKernels& out, std::string& err) {
+bool jit_compiled(const std::vector<int>& ids_in, bool bulk) {
+    std::vector<int> ids = ids_in;
+    const std::string key = id_key(ids, bulk);
+    std::lock_guard<std::mutex> lk(g_mu);
+    return ids.empty() || g_cubins.count(key);
+}
+
+int jit_kernels(const std::vector<int>& ids_in, JitKernels& out, std::string& err, bool bulk) {
     out = JitKernels();
     if (ids_in.empty()) return FDOG_OK;
     std::vector<int> ids = ids_in;
-    const std::string key = id_key(ids);
+    const std::string key = id_key(ids, bulk);
     {
         std::lock_guard<std::mutex> lk(g_mu);
         auto it = g_modules.find(key);
         if (it != g_modules.end()) { out = it->second; return FDOG_OK; }
     }
-    int rc = compile_module(ids, key, err);
+    int rc = compile_module(ids, key, bulk, err);
     if (rc != FDOG_OK) return rc;
     std::lock_guard<std::mutex> lk(g_mu);
     auto it = g_modules.find(key);
@@ -351,29 +352,29 @@ int jit_kernels(const std::vector<int>& ids_in, JitKernels& out, std::string& er
         err = std::string("cudaLibraryLoadData: ") + cudaGetErrorString(e);
         return FDOG_ECUDA;
     }
-    const char* names[6] = {"fdog_jit_fwd", "fdog_jit_bwd", "fdog_jit_mm", "fdog_jit_eval", "fdog_bulk_fwd",
-                            "fdog_bulk_bwd"};
+    const char* names[4] = {"fdog_jit_fwd", "fdog_jit_bwd", "fdog_jit_mm", "fdog_jit_eval"};
+    const char* bulk_names[2] = {"fdog_bulk_fwd", "fdog_bulk_bwd"};
     JitKernels kk;
-    for (int m = 0; m < 6; ++m) {
+    for (int m = 0; m < (bulk ? 2 : 4); ++m) {
         cudaKernel_t kern = nullptr;
-        e = cudaLibraryGetKernel(&kern, lib, names[m]);
+        e = cudaLibraryGetKernel(&kern, lib, bulk ? bulk_names[m] : names[m]);
         if (e != cudaSuccess) {
             cudaGetLastError();
             err = std::string("cudaLibraryGetKernel: ") + cudaGetErrorString(e);
             return FDOG_ECUDA;
         }
-        (m < 4 ? kk.fn[m] : kk.bulk[m - 4]) = reinterpret_cast<const void*>(kern);
+        kk.fn[m] = reinterpret_cast<const void*>(kern);
     }
     g_modules.emplace(key, kk);  // the library stays loaded for the life of the process
     out = kk;
     return FDOG_OK;
 }
 
-std::string jit_source(const std::vector<int>& ids_in) {
+std::string jit_source(const std::vector<int>& ids_in, bool bulk) {
     std::vector<int> ids = ids_in;
-    id_key(ids);
+    id_key(ids, bulk);
     std::lock_guard<std::mutex> lk(g_mu);
-    return generate_module(ids);
+    return generate_module(ids, bulk);
 }
 
 }  // namespace fdog

@@ -12,6 +12,7 @@
 #define FDOG_INF __int_as_float(0x7f800000)
 #define FDOG_FULL 0xffffffffu
 
+#ifdef FDOG_DISPATCH
 // largest instance index i with prefix[i] <= g, g the same in every lane
 __device__ __forceinline__ int fdog_find_inst(const int32_t* __restrict__ prefix, int n, int g, int lane) {
     if (n == 1) return 0;
@@ -113,7 +114,9 @@ extern "C" __global__ void __launch_bounds__(256) fdog_jit_fwd(SweepArgs a) { fd
 extern "C" __global__ void __launch_bounds__(256) fdog_jit_bwd(SweepArgs a) { fdog_jit_sweep<1>(a); }
 extern "C" __global__ void __launch_bounds__(256) fdog_jit_mm(SweepArgs a) { fdog_jit_sweep<2>(a); }
 extern "C" __global__ void __launch_bounds__(256) fdog_jit_eval(SweepArgs a) { fdog_jit_sweep<3>(a); }
+#endif
 
+#ifdef FDOG_BULK_DISPATCH
 // ---- bulk sweeps -------------------------------------------------------------
 // Update passes of one large instance.  In the sweeps above a warp waits in
 // turn for its tile's descriptor, its multipliers and ids, the terms they
@@ -304,3 +307,4 @@ __device__ __forceinline__ void fdog_bulk_sweep(const BulkArgs& a) {
 
 extern "C" __global__ void __launch_bounds__(256) fdog_bulk_fwd(BulkArgs a) { fdog_bulk_sweep<0>(a); }
 extern "C" __global__ void __launch_bounds__(256) fdog_bulk_bwd(BulkArgs a) { fdog_bulk_sweep<1>(a); }
+#endif

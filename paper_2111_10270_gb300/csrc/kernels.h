@@ -73,6 +73,7 @@ struct FlatArgsS {
 // Bulk sweeps of one instance (bulk.cu).
 struct BulkPlan {
     bool ready = false;
+    const void* fn[2] = {nullptr, nullptr};  // ascending, descending pass
     BulkArgs args{};
     int blocks_per_sm = 0;
 };
