@@ -144,28 +144,66 @@ extern "C" __global__ void __launch_bounds__(256) fdog_jit_eval(SweepArgs a) { f
 // warps fit an SM, and more stages take L1 from the gathers of T.  Capping the
 // registers at 48 for a fifth block made them spill (74.9 ms).  The L2 window
 // on T is worth 1 ms.
+// <ptx>
+__device__ __forceinline__ void fdog_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void fdog_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// the bulk copies that follow read what kernels wrote
+__device__ __forceinline__ void fdog_copies_see_kernels() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
 __device__ __forceinline__ unsigned fdog_smem_addr(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
 
-// waits for a stage's copies; gives up (false) after a second
-__device__ __forceinline__ bool fdog_bulk_wait(unsigned bar, unsigned parity) {
-    unsigned long long t0 = 0, t;
-    for (;;) {
-        unsigned done;
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return true;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-        if (t0 == 0) t0 = t;
-        else if (t - t0 > 1000000000ull) return false;
-    }
+__device__ __forceinline__ void fdog_bar_init(unsigned bars, int n) {
+    for (int s = 0; s < n; ++s)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * s) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+__device__ __forceinline__ void fdog_bar_expect(unsigned bar, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ bool fdog_bar_done(unsigned bar, unsigned parity) {
+    unsigned done;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+
+__device__ __forceinline__ unsigned long long fdog_now() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
 }
 
 __device__ __forceinline__ void fdog_bulk_copy(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+// </ptx>
+
+// waits for a stage's copies; gives up (false) after a second
+__device__ __forceinline__ bool fdog_bulk_wait(unsigned bar, unsigned parity) {
+    unsigned long long t0 = 0;
+    while (!fdog_bar_done(bar, parity)) {
+        const unsigned long long t = fdog_now();
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > 1000000000ull) return false;
+    }
+    return true;
+}
+
+// waits once more for up to `stages` of the `left` tiles' copies, from stage s of phase `parity` on
+__device__ __noinline__ void fdog_bulk_drain(unsigned bars, int stages, int s, unsigned parity, int left) {
+    for (int q = 0; q < stages && q < left; ++q) {
+        fdog_bulk_wait(bars + 8u * s, parity);
+        if (++s == stages) {
+            s = 0;
+            parity ^= 1u;
+        }
+    }
 }
 
 // (s, c) <- (s, c) + (x, y) for compensated FP32 pairs, as the butterflies above form them
@@ -182,25 +220,23 @@ __device__ __forceinline__ void fdog_bulk_sweep(const BulkArgs& a) {
     extern __shared__ __align__(128) float fdog_stages[];
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    fdog_pdl_trigger();
     // this warp's rows: stages; a table of the 32 tiles around the current one (16 ahead are filled in at a time, a
     // lane per tile, so that finding a tile costs next to nothing); the terms of four tiles; the barriers
     float* const stage0 = fdog_stages + (threadIdx.x >> 5) * FDOG_BULK_WARP_ROWS(a.stages, a.rows) * 32;
     int4* const tab = (int4*)(stage0 + a.stages * a.rows * 32);
     float* const terms = (float*)(tab + 32);
     const unsigned bars = fdog_smem_addr(terms + 136);
-    if (lane == 0) {
-        for (int s = 0; s < a.stages; ++s)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * s) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (lane == 0) fdog_bar_init(bars, a.stages);
     __syncwarp();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("fence.proxy.async.global;" ::: "memory");  // the copies read what kernels wrote
+    fdog_pdl_wait();
+    fdog_copies_see_kernels();
     const InstDev* __restrict__ I = a.inst;
     InstCtl* const ctl = I->ctl;
-    if (FDOG_INACTIVE(ctl)) return;
-    const bool zero = MODE == 0 && ctl->t_zero;  // a descending pass follows an ascending one
+    // all of it asked for at once; after an error no later pass waits again
+    const int done = ctl->done, iter = ctl->iter, limit = ctl->iter_limit, error = ctl->error, t_zero = ctl->t_zero;
+    if ((done != 0) | (iter >= limit) | (error != 0)) return;
+    const bool zero = MODE == 0 && t_zero;  // a descending pass follows an ascending one
     const float omega = I->omega;
     float* const lam0 = I->lam;
     const float* const cv0 = I->cv;
@@ -228,14 +264,14 @@ __device__ __forceinline__ void fdog_bulk_sweep(const BulkArgs& a) {
         }
         __syncwarp();
     };
+    bool late = false;
     auto issue = [&](int it, int s) {
-        if (it < n && lane == 0) {
+        if (it < n && lane == 0 && !late) {
             const int4 e = tab[it & 31];
             const unsigned rows = e.z & 31, more = (e.z >> 5 & 31) + (e.z >> 10 & 31);
             const unsigned bar = bars + 8u * s;
             const unsigned dst = fdog_smem_addr(stage0 + s * a.rows * 32);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((rows + more) * 128u)
-                         : "memory");
+            fdog_bar_expect(bar, (rows + more) * 128u);
             fdog_bulk_copy(dst, lam0 + e.x, rows * 128u, bar);
             fdog_bulk_copy(dst + rows * 128u, cv0 + e.y * 32, more * 128u, bar);
         }
@@ -245,7 +281,6 @@ __device__ __forceinline__ void fdog_bulk_sweep(const BulkArgs& a) {
     unsigned pk[8], plain_of = 0;
     int have = -1, s = 0;
     unsigned parity = 0;
-    bool late = false;
     for (int i = 0; i < n; ++i) {
         if ((i & 15) == 0) fill((i >> 4) + 1);
         const int4 e = tab[i & 31];
@@ -266,10 +301,12 @@ __device__ __forceinline__ void fdog_bulk_sweep(const BulkArgs& a) {
         const float* const sc = sl + (k - (e.z >> 15 & 15)) * 32;
         const int* const sv = (const int*)(sl + (k + (e.z >> 5 & 31) - (e.z >> 19 & 15)) * 32);
         // a lane that has waited in vain reports it (the host then returns an error) and waits no more; every lane
-        // goes on, so that the warp stays together
+        // goes on, so that the warp stays together.  No copy is started any more, and the lane that starts them waits
+        // once more for each that may still be on its way into this block's shared memory.
         if (!late && !fdog_bulk_wait(bars + 8u * s, parity)) {
             late = true;
             ctl->error = 1;
+            if (lane == 0) fdog_bulk_drain(bars, a.stages, s, parity, n - i);
         }
         float term = 0.f;
         FDOG_BULK_DISPATCH(MODE)
