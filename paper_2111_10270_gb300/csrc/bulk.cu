@@ -120,14 +120,18 @@ void plan_bulk(Decomposition& d, const uint16_t* local_ent) try {
         uint32_t local = 0, other = 0;  // layers
         std::vector<uint8_t> seen(np + 1, 0);
         for (; t < t1 && d.tiles[t].shape == shape; ++t) {
-            r.n_bdds += d.tiles[t].n_valid;
-            const int p = d.tiles[t].pattern;
-            if (seen[p + 1]) continue;
-            seen[p + 1] = 1;
+            const int p = d.tiles[t].pattern, valid = d.tiles[t].n_valid;
+            r.n_bdds += valid;
+            if (valid == kTile) {
+                if (seen[p + 1]) continue;
+                seen[p + 1] = 1;
+            }
+            // lanes without a BDD, in a run's last tile, need neither
+            const uint32_t lanes = valid == kTile ? 0xFFFFFFFFu : (1u << valid) - 1u;
             for (int l = 0; l < k; ++l) {
                 const uint32_t m = p < 0 ? 0xFFFFFFFFu : rest[static_cast<size_t>(p) * kEpiMaxK + l];
-                if (m != 0u) other |= 1u << l;
-                if (m != 0xFFFFFFFFu) local |= 1u << l;
+                if (m & lanes) other |= 1u << l;
+                if (~m & lanes) local |= 1u << l;
             }
         }
         auto range = [&](uint32_t m, int32_t& lo, int32_t& n) {

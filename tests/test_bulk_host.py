@@ -234,3 +234,17 @@ def test_a_copy_that_does_not_land_in_time(sweep, mode, hold_from):
 def test_no_pass_after_an_error(sweep):
     r = sweep(0, error=1)
     assert r["started"] == 0 and r["error"] == 1
+
+
+@pytest.mark.parametrize("labels,h,w,rows", [(4, 30, 32, 10), (4, 30, 31, 10), (4, 31, 31, 10), (8, 17, 19, 18), (8, 17, 18, 18)])
+def test_rows_copied_for_a_partial_last_tile(P, view, labels, h, w, rows):
+    """Marginalisation rows of L + 1 layers: L targets and the id of the layer shared with other edges, whether or not
+    the edges fill the last tile."""
+    inst = planned(P, ilpgen.mrf_grid(h, w, labels, 3), planner=1)
+    edges = h * (w - 1) + w * (h - 1)
+    v = view(inst)
+    assert v["rows"] == rows == (labels + 1) + labels + 1
+    tiles = -(-edges * 2 * labels // 32)
+    node_tiles = -(-h * w // 32)
+    # cv: targets and one id a marginalisation tile; the node rows have no local variable
+    assert v["cv_rows"] == tiles * (labels + 1) + node_tiles * labels
