@@ -631,6 +631,9 @@ int build_instance(fdog_instance* inst, int32_t device, void* cuda_stream, bool 
             if ((rc = plan_for_build(inst)) != FDOG_OK) return rc;
         }
     }
+    // a plan that a server made, which runs none
+    Decomposition& d = inst->dec;
+    if (bulk_wanted(inst) && !d.bulk_planned && !d.on_device && bulk_possible(d)) plan_bulk(d, d.local_ent.data());
     const std::vector<int> bulk = bulk_ids(inst);
     std::string unused;
     if (!bulk.empty() && jit_kernels(bulk, inst->bulk_jit, unused, true) != FDOG_OK) inst->dec.bulk_runs.clear();

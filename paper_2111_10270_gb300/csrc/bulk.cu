@@ -75,6 +75,7 @@ bool bulk_possible(const Decomposition& d) {
 
 // Without memory for it the instance runs the ordinary sweeps.
 void plan_bulk(Decomposition& d, const uint16_t* local_ent) try {
+    d.bulk_planned = true;
     d.bulk_runs.clear();
     d.bulk_pairs.clear();
     const size_t np = d.patterns.size() / 2;

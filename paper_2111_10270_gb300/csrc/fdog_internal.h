@@ -281,6 +281,7 @@ struct Decomposition {
     int64_t n_bdds = 0, n_slots = 0, n_nodes = 0, slots_pad = 0;
     int64_t n_work = 0, n_wpos = 0, n_local_ent = 0;  // sizes of work, wpos, local_ent
     // bulk sweeps (plan_bulk); empty: none
+    bool bulk_planned = false;
     std::vector<BulkRun> bulk_runs;
     std::vector<uint32_t> bulk_pairs;
     int32_t bulk_rows = 0;

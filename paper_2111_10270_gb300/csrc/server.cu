@@ -270,16 +270,18 @@ int fdog_server_submit(fdog_server* s, fdog_instance* inst, uint64_t* ticket) {
     if (!j) return FDOG_ENOMEM;
     j->inst = inst;
     inst->bulk_off = true;
+    auto refuse = [&](int code) {
+        inst->bulk_off = false;  // it stays the caller's
+        delete j;
+        return code;
+    };
     if (!inst->planned && inst->params.planner != 1) {
         // planned by the worker at admission, on the device where the builder takes it
         j->plan_on_admit = true;
         j->bytes = device_plan_bytes_bound(inst);
         j->t_submit = now_s();
         std::lock_guard<std::mutex> lk(s->mu);
-        if (s->fatal != FDOG_OK) {
-            delete j;
-            return s->fatal;
-        }
+        if (s->fatal != FDOG_OK) return refuse(s->fatal);
         j->ticket = s->next_ticket++;
         s->jobs.emplace(j->ticket, j);
         s->queue.push_back(j);
@@ -289,17 +291,11 @@ int fdog_server_submit(fdog_server* s, fdog_instance* inst, uint64_t* ticket) {
     }
     // host planning in the caller's thread, and the specialised kernels
     int rc = plan(inst, false);
-    if (rc != FDOG_OK) {
-        delete j;
-        return rc;
-    }
+    if (rc != FDOG_OK) return refuse(rc);
     std::vector<int> ids = jit_ids(inst), added;
     {
         std::lock_guard<std::mutex> lk(s->mu);
-        if (s->fatal != FDOG_OK) {
-            delete j;
-            return s->fatal;
-        }
+        if (s->fatal != FDOG_OK) return refuse(s->fatal);
         for (int id : ids)
             if (std::find(s->jit_universe.begin(), s->jit_universe.end(), id) == s->jit_universe.end()) {
                 s->jit_universe.push_back(id);
@@ -317,8 +313,7 @@ int fdog_server_submit(fdog_server* s, fdog_instance* inst, uint64_t* ticket) {
             for (int id : added)
                 s->jit_universe.erase(std::find(s->jit_universe.begin(), s->jit_universe.end(), id));
             inst->last_error = why;
-            delete j;
-            return rc;
+            return refuse(rc);
         }
     }
     j->bytes = static_cast<int64_t>(arena_size(inst));

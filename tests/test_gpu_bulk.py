@@ -4,6 +4,7 @@ import threading
 import pytest
 
 import ilpgen
+from bulk_view import compile_view
 
 pytestmark = pytest.mark.gpu
 
@@ -19,6 +20,11 @@ def P():
     import paper_2111_10270_gb300 as fdog
 
     return fdog
+
+
+@pytest.fixture(scope="module")
+def view(P, tmp_path_factory):
+    return compile_view(P, str(tmp_path_factory.mktemp("view")))
 
 
 def grid(P, h, w, labels, **kw):
@@ -52,3 +58,21 @@ def test_instances_of_common_kernels_on_two_threads(P):
         t.join()
     assert errors == []
     assert [g[1] for g in got] == [w[1] for w in want]
+
+
+def test_an_instance_back_from_a_server(P, view):
+    """A server runs the ordinary sweeps; built again by its owner, the instance runs those it would have without."""
+    import numpy as np
+
+    for planner in (0, 1):
+        inst = grid(P, 40, 41, 8, planner=planner)
+        server = P.Server(max_iters=20)
+        ticket = server.submit(inst)
+        assert server.wait(ticket)
+        inst = server.take(ticket)
+        server.close()
+        other = grid(P, 40, 41, 8, planner=planner).build(0)
+        inst.build(0)
+        assert view(other)["ready"] and view(inst)["ready"]
+        assert inst.iterate(20) == other.iterate(20)
+        assert np.array_equal(inst.multipliers()[2], other.multipliers()[2])
