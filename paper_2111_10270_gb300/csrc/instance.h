@@ -144,6 +144,8 @@ void free_device_plan(Decomposition& d, cudaStream_t s);
 int ensure_host_plan(fdog_instance* inst);
 size_t arena_size(const fdog_instance* inst);
 int fail_cuda(fdog_instance* inst, cudaError_t e, const char* where);
+using DeviceAlloc = cudaError_t (*)(void**, size_t);
+inline cudaError_t device_alloc(void** p, size_t bytes) { return cudaMalloc(p, bytes); }
 cudaError_t copy_async(fdog_instance* inst, void* dst, const void* src, size_t bytes, cudaMemcpyKind kind);
 int read_ctl(fdog_instance* inst, InstCtl& out);
 int addback(fdog_instance* inst);
@@ -163,6 +165,6 @@ cudaError_t launch_shard_init(fdog_instance* inst);
 // the instance's slots (slots.cu): arrays of n_slots entries to the caller's host memory (any may be null);
 // on return they are complete.  free_slots releases what the first read made.
 int read_slots(fdog_instance* inst, int32_t* var, int32_t* row, const float* dev0, float* out0, const float* dev1,
-               float* out1);
+               float* out1, DeviceAlloc alloc = device_alloc);
 void free_slots(fdog_instance* inst);
 }  // namespace fdog

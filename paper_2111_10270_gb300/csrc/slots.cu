@@ -9,7 +9,8 @@
 // slot, the reads of a tile within its own lines).  Up to kFewSlots slots, all
 // arrays are gathered by one launch and brought back by one copy, since there
 // every launch and copy counts more than the bytes; beyond, one array at a
-// time, so that the device holds one listed array only.
+// time, so that the device holds one listed array only.  On a device without
+// room for that one, the padded arrays are copied and listed on the host.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -71,7 +72,7 @@ void touch_pages(void* const* dst, int lists, size_t bytes) {
     });
 }
 
-int make_slots(fdog_instance* inst) {
+int make_slots(fdog_instance* inst, DeviceAlloc alloc) {
     if (inst->slot_first) return FDOG_OK;
     const Decomposition& d = inst->dec;
     const size_t nt = d.tiles.size(), nb = static_cast<size_t>(d.n_bdds);
@@ -88,12 +89,13 @@ int make_slots(fdog_instance* inst) {
         first[t] = at;
         at += d.tiles[t].n_valid * d.shapes[d.tiles[t].shape].k;
     }
-    char* p = nullptr;
+    void* at_dev = nullptr;
     const size_t bytes = up(nt) + up(nb) + up(ns);
-    if (cudaMalloc(reinterpret_cast<void**>(&p), bytes) != cudaSuccess) {
+    if (alloc(&at_dev, bytes) != cudaSuccess) {
         cudaGetLastError();
         return FDOG_ENOMEM;
     }
+    char* const p = static_cast<char*>(at_dev);
     int32_t* const d_first = reinterpret_cast<int32_t*>(p);
     int32_t* const d_row = reinterpret_cast<int32_t*>(p + up(nt));
     // a device-built plan's rows are on the device until a host call downloads the plan; from here on in slot_row
@@ -117,13 +119,48 @@ int make_slots(fdog_instance* inst) {
     return FDOG_OK;
 }
 
+// The same without device memory.
+int read_slots_on_host(fdog_instance* inst, int32_t* var, int32_t* row, const float* const (&dev)[2],
+                       float* const (&out)[2]) {
+    const int rc = ensure_host_plan(inst);
+    if (rc != FDOG_OK) return rc;
+    const Decomposition& d = inst->dec;
+    // each slot's place in the listed order and in the padded arrays, and its BDD
+    auto each = [&](auto&& put) {
+        int64_t q = 0;
+        for (const TileDev& t : d.tiles) {
+            const int k = d.shapes[t.shape].k;
+            for (int l = 0; l < t.n_valid; ++l)
+                for (int layer = 0; layer < k; ++layer)
+                    put(q++, t.slot_base + static_cast<int64_t>(layer) * kTile + l, t.bdd_base + l);
+        }
+    };
+    if (var) each([&](int64_t q, int64_t p, int32_t) { var[q] = d.var[p]; });
+    if (row) each([&](int64_t q, int64_t, int32_t b) { row[q] = d.bdd_row[b]; });
+    std::vector<float> h;
+    for (int a = 0; a < 2; ++a) {
+        if (!out[a]) continue;
+        try {
+            h.resize(static_cast<size_t>(d.slots_pad));
+        } catch (const std::bad_alloc&) {
+            return FDOG_ENOMEM;
+        }
+        cudaError_t e = copy_async(inst, h.data(), dev[a], sizeof(float) * h.size(), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(inst->stream);
+        if (e != cudaSuccess) return fail_cuda(inst, e, "copy slots");
+        each([&](int64_t q, int64_t p, int32_t) { out[a][q] = h[p]; });
+    }
+    return FDOG_OK;
+}
+
 }  // namespace
 
 int read_slots(fdog_instance* inst, int32_t* var, int32_t* row, const float* dev0, float* out0, const float* dev1,
-               float* out1) {
+               float* out1, DeviceAlloc alloc) {
     const Decomposition& d = inst->dec;
     if (d.n_slots == 0) return FDOG_OK;
-    int rc = make_slots(inst);
+    int rc = make_slots(inst, alloc);
+    if (rc == FDOG_ENOMEM) return read_slots_on_host(inst, var, row, {dev0, dev1}, {out0, out1});
     if (rc != FDOG_OK) return rc;
     const int32_t n = static_cast<int32_t>(d.n_slots);
     const size_t bytes = sizeof(int32_t) * static_cast<size_t>(n);

@@ -1,5 +1,5 @@
-"""What an instance's plan of bulk sweeps looks like from inside the library: a few lines of C++ over the internal
-headers, compiled beside it."""
+"""The library from inside: an instance's plan of bulk sweeps, and calls with a fake allocation.  A few lines of C++
+over the internal headers, compiled beside it."""
 import ctypes
 import os
 import subprocess
@@ -19,6 +19,12 @@ extern "C" void bulk_view(const fdog_instance* inst, long long* v) {
         if (s.jit >= 0) ids.push_back(s.jit);
     v[4] = fdog::jit_compiled(ids, false);
     v[5] = !ids.empty() && fdog::jit_compiled(ids, true);
+}
+
+// the slots read on a device that has no memory left
+extern "C" int read_on_full_device(fdog_instance* inst, int32_t* var, int32_t* row, float* lam) {
+    return fdog::read_slots(inst, var, row, inst->dev.lam, lam, nullptr, nullptr,
+                            [](void**, size_t) { return cudaErrorMemoryAllocation; });
 }
 """
 
@@ -40,4 +46,5 @@ def compile_view(P, folder):
         so.bulk_view(inst._h, v)
         return dict(zip(("runs", "rows", "cv_rows", "ready", "compiled", "bulk_compiled"), v))
 
+    view.so = so
     return view

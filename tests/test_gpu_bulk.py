@@ -1,4 +1,5 @@
 """GPU tests of the bulk sweeps' plan and of what instances that run them share."""
+import ctypes
 import threading
 
 import pytest
@@ -76,3 +77,21 @@ def test_an_instance_back_from_a_server(P, view):
         assert view(other)["ready"] and view(inst)["ready"]
         assert inst.iterate(20) == other.iterate(20)
         assert np.array_equal(inst.multipliers()[2], other.multipliers()[2])
+
+
+@pytest.mark.parametrize("planner", [0, 1], ids=["device plan", "host plan"])
+@pytest.mark.parametrize("size", [(9, 7, 3), (60, 61, 5)])
+def test_slots_are_read_on_a_full_device(P, view, size, planner):
+    """Without device memory for the listed order the host lists the slots, in the same order."""
+    import numpy as np
+
+    inst = grid(P, *size, planner=planner).build(0)
+    inst.iterate(7)
+    n = inst.info()["n_slots"]
+    var, row, lam = np.zeros(n, np.int32), np.zeros(n, np.int32), np.zeros(n, np.float32)
+    before = inst.info()["device_bytes"]
+    ptr = [ctypes.c_void_p(a.ctypes.data) for a in (var, row, lam)]
+    assert view.so.read_on_full_device(inst._h, *ptr) == P.FDOG_OK
+    assert inst.info()["device_bytes"] == before
+    for got, want in zip((var, row, lam), inst.multipliers()):
+        assert np.array_equal(got, want)
