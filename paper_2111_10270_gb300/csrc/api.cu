@@ -293,6 +293,33 @@ int ensure_host_plan(fdog_instance* inst) {
     return FDOG_OK;
 }
 
+// One allocation for every device array of the instance.  Where it fails with the arrays of bulk sweeps, about
+// a seventh more than without, the instance does without them.
+int allocate_arena(fdog_instance* inst, DeviceAlloc alloc) {
+    for (;;) {
+        std::vector<Item> items = arena_items(inst, inst->dev);
+        size_t total = 0;
+        std::vector<size_t> offs(items.size());
+        for (size_t q = 0; q < items.size(); ++q) {
+            offs[q] = total;
+            total = align_up(total + items[q].bytes, 256);
+        }
+        if (alloc(&inst->arena, total) == cudaSuccess) {
+            inst->arena_bytes = total;
+            for (size_t q = 0; q < items.size(); ++q) *items[q].ptr = static_cast<char*>(inst->arena) + offs[q];
+            return FDOG_OK;
+        }
+        cudaGetLastError();
+        inst->arena = nullptr;
+        if (bulk_ids(inst).empty()) {
+            inst->last_error = "cudaMalloc of " + std::to_string(total) + " bytes failed";
+            return FDOG_ENOMEM;
+        }
+        inst->dec.bulk_runs.clear();
+        inst->dec.bulk_planned = false;  // a later build may have the room
+    }
+}
+
 // Lay out every device array of the instance inside one allocation.
 int allocate_and_upload(fdog_instance* inst) {
     Decomposition& d = inst->dec;
@@ -302,22 +329,9 @@ int allocate_and_upload(fdog_instance* inst) {
     const int64_t nchunks = std::max<int64_t>(1, (nt + kLbChunk - 1) / kLbChunk);
     const int64_t nobj = std::max<int64_t>(1, (n + kObjChunk - 1) / kObjChunk);
     DevArrays& a = inst->dev;
-    std::vector<Item> items = arena_items(inst, a);
-    size_t total = 0;
-    std::vector<size_t> offs(items.size());
-    for (size_t q = 0; q < items.size(); ++q) {
-        offs[q] = total;
-        total = align_up(total + items[q].bytes, 256);
-    }
-    cudaError_t e = cudaMalloc(&inst->arena, total);
-    if (e != cudaSuccess) {
-        inst->arena = nullptr;
-        inst->last_error = "cudaMalloc of " + std::to_string(total) + " bytes failed";
-        cudaGetLastError();
-        return FDOG_ENOMEM;
-    }
-    inst->arena_bytes = total;
-    for (size_t q = 0; q < items.size(); ++q) *items[q].ptr = static_cast<char*>(inst->arena) + offs[q];
+    const int rc = allocate_arena(inst, device_alloc);
+    if (rc != FDOG_OK) return rc;
+    cudaError_t e = cudaSuccess;
 
     // descriptor
     InstDev h{};

@@ -134,6 +134,10 @@ struct fdog_instance {
 };
 
 namespace fdog {
+// how device memory is allocated
+using DeviceAlloc = cudaError_t (*)(void**, size_t);
+inline cudaError_t device_alloc(void** p, size_t bytes) { return cudaMalloc(p, bytes); }
+
 int plan(fdog_instance* inst, bool compile_jit = true);
 // device builder (plan_device.cu): FDOG_OK, plan_leave_to_host() when the
 // instance needs the host builder, or an FDOG_* error
@@ -143,9 +147,8 @@ void free_device_plan(Decomposition& d, cudaStream_t s);
 // downloads the arrays of a device-built plan that host calls read
 int ensure_host_plan(fdog_instance* inst);
 size_t arena_size(const fdog_instance* inst);
+int allocate_arena(fdog_instance* inst, DeviceAlloc alloc);
 int fail_cuda(fdog_instance* inst, cudaError_t e, const char* where);
-using DeviceAlloc = cudaError_t (*)(void**, size_t);
-inline cudaError_t device_alloc(void** p, size_t bytes) { return cudaMalloc(p, bytes); }
 cudaError_t copy_async(fdog_instance* inst, void* dst, const void* src, size_t bytes, cudaMemcpyKind kind);
 int read_ctl(fdog_instance* inst, InstCtl& out);
 int addback(fdog_instance* inst);

@@ -7,6 +7,8 @@ import subprocess
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 SOURCE = r"""
+#include <cstdlib>
+#include "../../include/fastdog.h"
 #include "instance.h"
 extern "C" void bulk_view(const fdog_instance* inst, long long* v) {
     const fdog::Decomposition& d = inst->dec;
@@ -19,6 +21,22 @@ extern "C" void bulk_view(const fdog_instance* inst, long long* v) {
         if (s.jit >= 0) ids.push_back(s.jit);
     v[4] = fdog::jit_compiled(ids, false);
     v[5] = !ids.empty() && fdog::jit_compiled(ids, true);
+}
+
+// one allocation for a planned instance on a device with room for `room` bytes (host memory here); what it took
+extern "C" int allocate_with_room(fdog_instance* inst, long long room, long long* bytes) {
+    static size_t limit;
+    limit = static_cast<size_t>(room);
+    const int rc = fdog::allocate_arena(inst, [](void** p, size_t n) {
+        if (n > limit) return cudaErrorMemoryAllocation;
+        *p = std::calloc(n, 1);
+        return cudaSuccess;
+    });
+    *bytes = rc == FDOG_OK ? static_cast<long long>(inst->arena_bytes) : 0;
+    std::free(inst->arena);
+    inst->arena = nullptr;
+    inst->dev = fdog::DevArrays();
+    return rc;
 }
 
 // the slots read on a device that has no memory left

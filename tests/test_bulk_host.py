@@ -37,6 +37,23 @@ def test_bulk_kernels_are_compiled_for_instances_that_run_them(P, view):
     assert v["runs"] > 0 and v["compiled"] and v["bulk_compiled"], v
 
 
+def test_a_device_without_room_for_bulk_sweeps(P, view):
+    """An instance that fits only without their arrays is laid out without."""
+    import ctypes
+
+    ilp = ilpgen.mrf_grid(17, 19, 8, 3)
+    inst, plain = planned(P, ilp), planned(P, ilp, block_threads=128)
+    with_bulk, without = inst.info()["device_bytes"], plain.info()["device_bytes"]
+    assert with_bulk > without
+    took = ctypes.c_longlong()
+    assert view.so.allocate_with_room(inst._h, ctypes.c_longlong(without - 1), ctypes.byref(took)) == P.capi.FDOG_ENOMEM
+    inst = planned(P, ilp)
+    assert view.so.allocate_with_room(inst._h, ctypes.c_longlong(with_bulk), ctypes.byref(took)) == P.FDOG_OK
+    assert took.value == with_bulk and view(inst)["runs"] > 0
+    assert view.so.allocate_with_room(inst._h, ctypes.c_longlong(with_bulk - 1), ctypes.byref(took)) == P.FDOG_OK
+    assert took.value == without == inst.info()["device_bytes"] and view(inst)["runs"] == 0
+
+
 # The kernel itself on the CPU: a warp as 32 threads, its PTX replaced by copies and barriers that the test controls.
 EMULATION = r"""
 #include <algorithm>
