@@ -44,6 +44,7 @@ struct Engine {
     LaunchCfg cfg;
     Profiler* prof = nullptr;  // optional kernel timing (graphs are not used while it is on)
     int chunk = 8;             // iterations per graph launch (set by view_autotune)
+    int dual_replays = 1;      // graph launches per scheduling step while no member rounds (set by view_autotune)
     std::vector<int> jit_universe;  // if set: the shape ids every view's specialised module covers
     InstStatus* dev_status = nullptr;
     InstStatus* host_status = nullptr;  // pinned
@@ -83,6 +84,7 @@ struct Member {
     int noconv = 0;
     int start_iter = 0;
     int dual_iters = 0;
+    int left = 0;  // iterations to the end of the running re-optimisation
 };
 
 // Prepares members [first, end) of `ms`: iteration budget max_iters (0: they
