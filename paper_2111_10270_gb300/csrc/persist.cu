@@ -92,7 +92,7 @@ __device__ __forceinline__ void sweep_pass(const SweepArgs (&c)[2], int n_reg, i
     // segmented tiles first: they are the longest walks
     for (int g = gw; g < n_seg + n_reg; g += nw) {
         const int gn = g + nw;
-        if (g < n_seg) seg_tile<2, MODE>(c[kSegClass], g, gn < n_seg ? gn : n_seg, wsm, lane);
+        if (g < n_seg) seg_tile<2, MODE, false>(c[kSegClass], g, gn < n_seg ? gn : n_seg, wsm, lane);
         else reg_tile<2, MODE>(c[kRegClass], g - n_seg, gn - n_seg, wsm, lane);
     }
 }

@@ -623,6 +623,10 @@ __global__ void __launch_bounds__(256) sweep_kernel(SweepArgs a) {
 // (ascending, descending) to 20.1 and 16.4; what is left of a warp's 1,640
 // instructions is a chain: 10.5 cycles each, 4 of them memory, 2.8 the
 // latency of the operation before, 1.6 instruction fetch.
+// Without AHEAD a segment is loaded when the one before it is done: the
+// persistent kernel (persist.cu), whose passes share 128 registers a thread,
+// spilled 816 bytes with the look-ahead and 484 without (39.8 instances/s in
+// place of 35.4 on 64 cell-tracking sequences).
 // Shared memory per warp: a.kstride checkpoints x W labels x 32 lanes, then
 // the tile-local staging (a.epi layers).
 // shared-memory floats one warp of seg_tile uses
@@ -631,7 +635,7 @@ __host__ __device__ __forceinline__ size_t seg_warp_floats(const SweepArgs& a) {
     return static_cast<size_t>(a.kstride) * W * kTile + static_cast<size_t>(a.epi) * kTile * 2;
 }
 
-template <int W, int MODE>
+template <int W, int MODE, bool AHEAD = true>
 __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, float* wsm, int lane) {
     constexpr int C = kRegK;
     constexpr bool update = MODE == kFwdUpdate || MODE == kBwdUpdate;
@@ -696,7 +700,7 @@ __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, 
     for (int u = nseg - 1; u >= 0; --u) {
         const int s = seg_of(u);
         const int kk = min(k - s * C, C);
-        if (u > 0) {  // in flight while this segment is swept
+        if (AHEAD && u > 0) {  // in flight while this segment is swept
             fetch_lam(seg_of(u - 1), Ln);
             load_segment_codes<W>(tpl, seg_of(u - 1) * C, cn);
         }
@@ -713,9 +717,12 @@ __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, 
                     if (j < kk) push_labels<W>(x, c[j], L[j]);
             }
         }
-        if (u > 0) {
+        if (AHEAD && u > 0) {
 #pragma unroll
             for (int j = 0; j < C; ++j) { L[j] = Ln[j]; c[j] = cn[j]; }
+        } else if (u > 0) {
+            fetch_lam(seg_of(u - 1), L);
+            load_segment_codes<W>(tpl, seg_of(u - 1) * C, c);
         }
     }
     float term = 0.f;
@@ -724,7 +731,7 @@ __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, 
     } else {
         if constexpr (update) {
             fetch_terms(seg_of(0), V, T);
-            if (nseg > 1) fetch_var(seg_of(1), V);
+            if (AHEAD && nseg > 1) fetch_var(seg_of(1), V);
         }
         float* __restrict__ mm0 = I->mm0;
         float* __restrict__ mm1 = I->mm1;
@@ -734,7 +741,7 @@ __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, 
         for (int u = 0; u < nseg; ++u) {
             const int s = seg_of(u);
             const int kk = min(k - s * C, C);
-            if (u + 1 < nseg) {  // in flight while this segment is swept
+            if (AHEAD && u + 1 < nseg) {  // in flight while this segment is swept
                 fetch_lam(seg_of(u + 1), Ln);
                 load_segment_codes<W>(tpl, seg_of(u + 1) * C, cn);
                 if constexpr (update) {
@@ -806,9 +813,16 @@ __device__ __forceinline__ void seg_tile(const SweepArgs& a, int g, int g_next, 
                     }
                 }
             }
-            if (u + 1 < nseg) {
+            if (AHEAD && u + 1 < nseg) {
 #pragma unroll
                 for (int j = 0; j < C; ++j) { L[j] = Ln[j]; T[j] = Tn[j]; c[j] = cn[j]; }
+            } else if (u + 1 < nseg) {
+                fetch_lam(seg_of(u + 1), L);
+                load_segment_codes<W>(tpl, seg_of(u + 1) * C, c);
+                if constexpr (update) {
+                    fetch_var(seg_of(u + 1), V);
+                    fetch_terms(seg_of(u + 1), V, T);
+                }
             }
         }
         if constexpr (!asc) term = fmaf(-omega, negsum, x[0]);
