@@ -6,6 +6,7 @@ import pytest
 
 import ilpgen
 from bulk_view import compile_view
+from test_gpu_sweep_tiles import BULK
 
 pytestmark = pytest.mark.gpu
 
@@ -95,3 +96,12 @@ def test_slots_are_read_on_a_full_device(P, view, size, planner):
     assert inst.info()["device_bytes"] == before
     for got, want in zip((var, row, lam), inst.multipliers()):
         assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("name", sorted(BULK))
+def test_the_cases_compared_with_ordinary_sweeps_run_bulk_sweeps(P, view, name):
+    """Those of test_bulk_sweeps_match_the_ordinary_ones, which only sees that memory was set aside."""
+    ilp = BULK[name]()
+    params = dict(tol=0.0, max_rounds=3, jit=1)
+    assert view(P.Instance.from_ilp(ilp, P.capi.default_params(**params)).build(0))["ready"]
+    assert not view(P.Instance.from_ilp(ilp, P.capi.default_params(block_threads=128, **params)).build(0))["ready"]
