@@ -8,6 +8,7 @@
 
 #include "instance.h"
 #include "kernels.h"
+#include "sweep.cuh"
 
 namespace fdog {
 
@@ -35,13 +36,9 @@ __global__ void __launch_bounds__(256) bulk_targets_kernel(const InstDev* insts,
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < total; w += warps) {
-        int lo = 0, hi = n_inst - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(prefix + mid) <= w) lo = mid; else hi = mid - 1;
-        }
-        const InstDev* __restrict__ I = insts + lo;
-        const int g = w - __ldg(prefix + lo) - I->bulk_first;
+        const int ii = dev::find_inst_warp(prefix, n_inst, w, lane);
+        const InstDev* __restrict__ I = insts + ii;
+        const int g = w - __ldg(prefix + ii) - I->bulk_first;
         if (!I->cv || g < 0 || g >= I->bulk_tiles) continue;
         int q = I->n_bulk_runs - 1;
         while (q > 0 && I->bulk_runs[q].tile > g) --q;

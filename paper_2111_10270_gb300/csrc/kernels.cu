@@ -33,7 +33,6 @@ namespace {
 
 using dev::FlatArgs;
 using dev::LbArgs;
-using dev::block_pair_reduce;
 using dev::CommitIn;
 using dev::commit_in;
 using dev::commit_iteration;
