@@ -33,6 +33,7 @@
 #include <chrono>
 #include <cstring>
 #include <limits>
+#include <new>
 #include <vector>
 
 #include "fdog_internal.h"
@@ -840,10 +841,16 @@ int plan_on_device(fdog_instance* inst, int jit_mode, bool fuse_local) {
     PLAN_CHECK(cudaGetLastError());
     PLAN_CHECK(cudaStreamSynchronize(st));
     if (bulk_wanted(inst) && bulk_possible(out)) {
-        std::vector<uint16_t> ent(static_cast<size_t>(out.n_local_ent));
-        PLAN_CHECK(cudaMemcpyAsync(ent.data(), out.d_local_ent, sizeof(uint16_t) * ent.size(), cudaMemcpyDeviceToHost, st));
-        PLAN_CHECK(cudaStreamSynchronize(st));
-        plan_bulk(out, ent.data());
+        std::vector<uint16_t> ent;
+        try {
+            ent.resize(static_cast<size_t>(out.n_local_ent));
+        } catch (const std::bad_alloc&) {  // no bulk sweeps
+        }
+        if (!ent.empty()) {
+            PLAN_CHECK(cudaMemcpyAsync(ent.data(), out.d_local_ent, sizeof(uint16_t) * ent.size(), cudaMemcpyDeviceToHost, st));
+            PLAN_CHECK(cudaStreamSynchronize(st));
+            plan_bulk(out, ent.data());
+        }
     }
     out.on_device = true;
     inst->plan_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
