@@ -17,11 +17,14 @@ namespace {
 constexpr int kBulkWarps = 8;
 constexpr int kBulkStages = 2;
 // The rule for bulk sweeps: three quarters of the tiles plain, and at least this many of them.  200 iterations on grids,
-// ms, ordinary and bulk sweeps: 4 labels, 0.28 k tiles 3.43 and 3.40, 2.1 k 4.31 and 3.91, 8.7 k 5.37 and 5.10, 18 k 7.25
-// and 6.40, 48 k 12.5 and 10.4; 8 labels, 0.56 k tiles 3.90 and 3.72, 4.2 k 5.97 and 4.82.  Rows of three layers
-// (2 labels) leave little to form from a copied tile: 4.2 k tiles 4.08 and 4.33, 10 k 5.05 and 5.13, 33 k 8.23 and 8.11,
-// 66 k 13.2 and 12.1.  With 3 labels the edges that a tile's end cuts make every tile a mixed one, whose slots all need
-// ids and whose layers take both ways: 31 k tiles 14.8 and 16.3.
+// ms, ordinary and bulk sweeps: 4 labels, 0.27 k tiles 3.13 and 3.07, 2.1 k 4.11 and 3.75, 8.6 k 5.10 and 4.81, 19 k 6.85
+// and 5.94, 48 k 12.1 and 10.1; 8 labels, 0.31 k tiles 3.50 and 3.33, 4.2 k 5.65 and 4.48.  Rows of three layers (2
+// labels) leave little to form from a copied tile: 4.8 k tiles 4.11 and 3.99, 11 k 4.87 and 4.91, 25 k 6.56 and 6.21,
+// 37 k 7.91 and 7.58, 74 k 12.9 and 11.7.  With 3 labels the edges that a tile's end cuts make every tile a mixed one,
+// whose slots all need ids and whose layers take both ways: 16 k tiles 6.32 and 6.43, 65 k 14.4 and 15.4 (and once 26).
+// So they do with 5 to 7 labels, where the longer rows can pay for it (9.8 k tiles of 5 labels 5.63 and 5.69, 26 k 9.65
+// and 8.89; 7.8 k of 6 labels 6.05 and 5.66): the rule leaves them on the ordinary sweeps.  Other families of this
+// repository have no tile-local variables in regular tiles.
 constexpr int32_t kBulkMinTiles = 256, kBulkMinShortTiles = 16384;
 constexpr int64_t kBulkMaxPatterns = 64;  // a tile's table entry has 8 bits for its pattern; more would be large tables
 

@@ -136,10 +136,12 @@ extern "C" __global__ void __launch_bounds__(256) fdog_jit_eval(SweepArgs a) { f
 // tile, instead of at the end of that pass: T is neither written nor gathered
 // for it, and its slots need no ids.  The same FP32 operations in the same
 // order, so the same terms.  A pass moves 274 MB, in about 48 us: the 500
-// iterations and two roundings of that grid went from 88.2 to 69.5 ms.  What
-// bounds it now is instructions, 281 and 304 a tile with 68% of the issue
-// slots taken (338 before tiles were looked up 16 at a time, the second copy
-// was merged, and plain patterns got a path without choices per slot).  Two
+// iterations and two roundings of that grid went from 88.2 to 69.2 ms.  What
+// bounds it now is instructions, 265 and 310 a tile (ascending, descending)
+// with 66 and 69% of the issue slots taken, before memory latency (3 to 4 of
+// the 10 to 11 cycles between two instructions of a warp).  Tiles are looked
+// up 16 at a time, both copies of a pair by one bulk copy, and plain patterns
+// have a path without choices per slot.  Two
 // stages (69.5 ms; three 70.3, four 74.5): at 62 registers four blocks of eight
 // warps fit an SM, and more stages take L1 from the gathers of T.  Capping the
 // registers at 48 for a fifth block made them spill (74.9 ms).  The L2 window

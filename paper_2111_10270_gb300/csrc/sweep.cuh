@@ -620,9 +620,9 @@ __global__ void __launch_bounds__(256) sweep_kernel(SweepArgs a) {
 // codes, multipliers and ids are each loaded at once, and one segment (of the
 // ids: two) ahead of their use, so that no walk waits for memory in the middle.
 // A lone cell-tracking sequence (160 tiles) went from 25.7 and 20.7 us
-// (ascending, descending) to 20.1 and 16.4; what is left of a warp's 1,640
-// instructions is a chain: 10.5 cycles each, 4 of them memory, 2.8 the
-// latency of the operation before, 1.6 instruction fetch.
+// (ascending, descending) to 20.1 and 16.4; what is left of a warp's 1,920 and
+// 1,720 instructions is a chain: 9.6 and 10.5 cycles each, 3.4 and 3.8 of them
+// memory, 3 the latency of the operation before, 1.6 instruction fetch.
 // Without AHEAD a segment is loaded when the one before it is done: the
 // persistent kernel (persist.cu), whose passes share 128 registers a thread,
 // spilled 816 bytes with the look-ahead and 484 without (39.8 instances/s in
