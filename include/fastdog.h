@@ -576,7 +576,7 @@ int fdog_shard_commit(fdog_instance* inst, double lb, int32_t* stop);
  * finite or the total is beyond the largest double.
  * dev_values (n doubles) and dev_out (one double) are device memory owned by
  * the caller; the call allocates nothing: its scratch is a static device
- * array of about 32 KiB that every GPU loading this library holds until the
+ * array of about 42 KiB that every GPU loading this library holds until the
  * process exits.  n = 0 writes `constant`.
  * n may be at most 8,388,608 (FDOG_EINVAL beyond, or for negative n or NULL
  * pointers).  The first call on a device looks up that array's device address

@@ -10,7 +10,7 @@
 // sum.  The sum is formed in integers, so that it is exact whatever the order:
 // a block aligns its values to the largest exponent among them and adds them as
 // 128-bit fixed-point numbers; a second launch of one block adds the blocks'
-// totals in the same way.  Bits that such a window has no place for (2^-112 of
+// totals in the same way.  Bits that such a window has no place for (2^-101 of
 // the largest value and below: values of very different size, which may be all
 // that is left once the large ones cancel) go through windows of their own into
 // an accumulator of the whole FP64 range.  What bounds it is
@@ -18,7 +18,9 @@
 // us: FP64 additions run at two per clock and SM on this part, so that the
 // compensated FP64 tree over 256 values per block that stood here took 144 us a
 // call for 4,000,037 values and 47 us for 2^20; integer shifts and additions run
-// at the full rate (22 and 14 us; 2,000 values 8.2, with the tree 11.2).
+// at the full rate (18.4 and 10.3 us; 2,000 values 6.2, with the tree 11.2).  The
+// blocks' totals travel as integers too: as pairs of doubles they and a second
+// launch that handles every case in line took 3 us more.
 // Scratch -- the blocks' totals and that accumulator -- is one file-scope static
 // device array instead of memory owned by an instance.  A call leaves nothing in
 // it that a later one reads: the second launch needs no counter of finished
@@ -44,12 +46,22 @@ constexpr int kMaxBlocks = static_cast<int>(kMaxValues / (kThreads * kManyPer));
 static_assert(kFewMax / (kThreads * kFewPer) <= kMaxBlocks, "scratch holds the totals of either kind");
 constexpr int kMaxDevices = 64;
 
+// Fixed-point sums.  A value of biased exponent e (1 for subnormal numbers) is
+// m 2^(e - 1075) with a 53-bit m; beside values of largest exponent emax it is
+// added as m 2^(kUp - (emax - e)), without the bits below the last place.  2^23
+// such terms (4,096 values a block, 2,048 blocks) and the sign fit 128 bits.
+constexpr int kUp = 49;
+struct __align__(16) Fixed {
+    unsigned long long lo, hi;  // two's complement
+};
+
 constexpr int kDigits = 70;
 struct Scratch {
-    double part[2 * kMaxBlocks];  // total of each block: leading part, remainder; zeros if it went into digit
-    // The blocks' totals that a window or a pair of doubles cannot hold, as digits of 32 bits in 64 from bit
-    // 2^-1134 on, summed by integer atomics.  Zero between calls: the finishing block, which runs after every
-    // block of its call, clears them, so the last call to finish does whatever overlapped before it.
+    Fixed part[kMaxBlocks];  // total of each block, zero if it went into digit
+    int exponent[kMaxBlocks];  // the exponent it is aligned to; 2047: a value was not finite
+    // The blocks' totals that a window cannot hold, as digits of 32 bits in 64 from bit 2^-1123 (2^(1 - 1075 - kUp))
+    // on, summed by integer atomics.  Zero between calls: the finishing block, which runs after every block of its
+    // call, clears them, so the last call to finish does whatever overlapped before it.
     unsigned long long digit[kDigits];
 };
 
@@ -62,15 +74,6 @@ std::mutex g_mu;
 // per device: the scratch address and the id of the context it was looked up in
 Scratch* g_addr[kMaxDevices] = {};
 unsigned long long g_ctx[kMaxDevices] = {};
-
-// Fixed-point sums.  A value of biased exponent e (1 for subnormal numbers) is
-// m 2^(e - 1075) with a 53-bit m; beside values of largest exponent emax it is
-// added as m 2^(kUp - (emax - e)), without the bits below the last place.  2^14
-// such terms and the sign fit 128 bits.
-constexpr int kUp = 60;
-struct Fixed {
-    unsigned long long lo, hi;  // two's complement
-};
 
 __device__ __forceinline__ int exponent_of(double v) {
     const int e = (__double2hiint(v) >> 20) & 0x7FF;
@@ -152,7 +155,7 @@ __device__ __noinline__ double round_digits(unsigned long long* digit) {
     m |= below >> 32;
     bool more = (below & mask) != 0;
     for (int i = top - 3; i >= 0 && !more; --i) more = digit[i] != 0;
-    const int e = 32 * top + 31 - lz - 1134;  // m 2^(e - 63)
+    const int e = 32 * top + 31 - lz - 1074 - kUp;  // m 2^(e - 63)
     const unsigned long long low = m & 0x7FFu;
     m >>= 11;
     if (low > 0x400u || (low == 0x400u && (more || (m & 1u)))) ++m;
@@ -221,7 +224,7 @@ __device__ __forceinline__ bool window_sum(double (&x)[N], int emax, Fixed& a) {
     return __syncthreads_or(rest);
 }
 
-// the block's values into digits, window by window (each takes 113 bits of exponent at least: at most 19)
+// the block's values into digits, window by window (each takes 102 bits of exponent at least: at most 21)
 template <int N>
 __device__ __forceinline__ void digits_of(double (&x)[N], unsigned long long* digit) {
     bool more = true;
@@ -287,36 +290,27 @@ __global__ void __launch_bounds__(kThreads, PER > 4 ? 4 : 8) bound_reduce_noallo
 #pragma unroll
     for (int q = 0; q < PER; ++q) add_key(k, x[q]);
     const int2 e = block_exponents(k);
-    double2 p = make_double2(0.0, 0.0);
-    if (e.y == 0x7FF) {  // a value is not finite
-        p.x = __longlong_as_double(0x7ff8000000000000ll);
-    } else if (e.y - e.x <= kUp) {
-        Fixed a{0, 0};
+    Fixed a{0, 0};
+    if (e.y < 0x7FF && e.y - e.x <= kUp) {
 #pragma unroll
         for (int q = 0; q < PER; ++q) add_value<true>(a, x[q], e.y);
         block_sum(a);
-        if (threadIdx.x == 0 && !to_pair(a, e.y, p)) {
-            add_digits(scr->digit, a, e.y);
-            p = make_double2(0.0, 0.0);
-        }
-    } else {
+    } else if (e.y < 0x7FF) {
         spread_block<PER>(v, n, scr->digit);
     }
     if (threadIdx.x == 0) {
-        scr->part[2 * blockIdx.x] = p.x;
-        scr->part[2 * blockIdx.x + 1] = p.y;
+        scr->part[blockIdx.x] = a;
+        scr->exponent[blockIdx.x] = e.y;
     }
 }
 
 // The rest of a sum that the finishing block could not form in one window: the blocks' totals, read again, and the
 // constant into digits, rounded once.  Out of line: the usual path is a few hundred instructions, which a lone block
 // waits for.
-__device__ __noinline__ void finish_digits(const double* part, int parts, double constant, double* out,
+__device__ __noinline__ void finish_digits(const Scratch* scr, int blocks, double constant, double* out,
                                            unsigned long long* digit) {
-    for (int at = 0; at < parts; at += kThreads) {
-        double x[1] = {at + static_cast<int>(threadIdx.x) < parts ? __ldcg(part + at + threadIdx.x) : 0.0};
-        digits_of(x, digit);
-    }
+    for (int b = threadIdx.x; b < blocks; b += kThreads) add_digits(digit, scr->part[b], scr->exponent[b]);
+    __syncthreads();
     if (threadIdx.x == 0) {
         const int e = exponent_of(constant);
         if (e == 0x7FF) {
@@ -331,24 +325,49 @@ __device__ __noinline__ void finish_digits(const double* part, int parts, double
 }
 
 // the blocks' totals and the constant, by one block
-__global__ void __launch_bounds__(kThreads) bound_finish_noalloc_kernel(Scratch* scr, int parts, double constant,
+__global__ void __launch_bounds__(kThreads) bound_finish_noalloc_kernel(Scratch* scr, int blocks, double constant,
                                                                          double* __restrict__ out) {
     __shared__ unsigned long long digit[kDigits];
+    __shared__ int most[kThreads / 32];
     __shared__ bool done;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const unsigned long long d = threadIdx.x < kDigits ? __ldcg(scr->digit + threadIdx.x) : 0ull;
-    Keys k;
-    for (int q = threadIdx.x; q < parts; q += kThreads) add_key(k, __ldcg(scr->part + q));
-    const int e = block_exponents(k).y;
+    const unsigned long long d = threadIdx.x < kDigits ? scr->digit[threadIdx.x] : 0ull;
+    int e = 1;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < blocks; b += kThreads) {
+        const Fixed a = scr->part[b];
+        const int eb = scr->exponent[b];
+        if ((a.lo | a.hi) != 0ull || eb == 0x7FF) e = max(e, eb);
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) most[threadIdx.x >> 5] = e;
     if (d) scr->digit[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) e = max(e, most[w]);
     if (e == 0x7FF) {
         if (threadIdx.x == 0) *out = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
+    // totals aligned to the largest exponent; what that would cut off goes another way
     Fixed t{0, 0};
     bool rest = d != 0;
-    for (int q = threadIdx.x; q < parts; q += kThreads)
-        rest = !is_zero(add_value<false>(t, __ldcg(scr->part + q), e)) || rest;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < blocks; b += kThreads) {
+        Fixed a = scr->part[b];
+        const int down = min(max(e - scr->exponent[b], 0), 127);  // less than 0: a zero
+        const int part = down & 63;
+        const unsigned long long sign = static_cast<long long>(a.hi) < 0 ? ~0ull : 0ull;
+        if (down >= 64) {
+            rest = rest || a.lo != 0;
+            a.lo = a.hi;
+            a.hi = sign;
+        }
+        rest = rest || (a.lo & ((1ull << part) - 1)) != 0;
+        a.lo = a.lo >> part | (a.hi << 1) << (63 - part);
+        a.hi = static_cast<unsigned long long>(static_cast<long long>(a.hi) >> part);
+        add(t, a);
+    }
     block_sum(t);
     rest = __syncthreads_or(rest);
     if (threadIdx.x == 0) {
@@ -361,7 +380,7 @@ __global__ void __launch_bounds__(kThreads) bound_finish_noalloc_kernel(Scratch*
     }
     if (threadIdx.x < kDigits) digit[threadIdx.x] = d;
     __syncthreads();
-    if (!done) finish_digits(scr->part, parts, constant, out, digit);
+    if (!done) finish_digits(scr, blocks, constant, out, digit);
 }
 
 // Unique id of the calling thread's current CUDA context (0 if there is
@@ -441,8 +460,8 @@ extern "C" int fdog_bound_reduce_noalloc(const double* dev_values, int64_t n, do
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
         // programmatic launch: its block waits on the device for the end of the launch above
-        int parts = 2 * static_cast<int>(blocks);
-        void* args[] = {&scr, &parts, &constant, &dev_out};
+        int n_blocks = static_cast<int>(blocks);
+        void* args[] = {&scr, &n_blocks, &constant, &dev_out};
         e = fdog::launch_windowed(reinterpret_cast<const void*>(bound_finish_noalloc_kernel), 1, kThreads, args, 0, s,
                                   fdog::L2Window());
         if (e != cudaSuccess) cudaGetLastError();

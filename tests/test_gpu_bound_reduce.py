@@ -89,6 +89,16 @@ def test_sums_of_every_size(env, n, kind):
         assert abs(got - want) <= math.ulp(want), (got, want)
 
 
+@pytest.mark.parametrize("apart", [0, 1, 48, 49, 50, 63, 64, 65, 101, 102, 103, 112, 127, 128, 129, 700])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_totals_of_blocks_far_apart(env, sign, apart):
+    """The first block's total and the others' at every distance of their exponents that an alignment treats apart."""
+    v = np.zeros(3 * 1024)
+    v[5], v[1024 + 7], v[2048 + 9] = sign * 2.0 ** apart, 1.0 + 2.0 ** -52, -2.0 ** -30
+    for constant in (0.0, -sign * 2.0 ** apart):
+        assert abs(total(env, v, constant) - exact(v, constant)) <= math.ulp(exact(v, constant))
+
+
 def test_totals_beyond_the_range(env):
     assert math.isnan(total(env, np.array([1.7e308, 1.7e308])))
     assert math.isnan(total(env, np.array([1.7e308, 1e-300]), 1.7e308))
