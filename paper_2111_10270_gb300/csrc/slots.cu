@@ -5,7 +5,7 @@
 // the caller's arrays get plain copies.  Copying the padded arrays and walking
 // them slot by slot on the host took 5.7 ms for the variables and rows and 2.8
 // ms for each value array of 5,484,544 slots, on top of 0.13 ms for the copy
-// itself; the gather takes about 10 us an array (it reads and writes 4 bytes a
+// itself; the gather takes about 16 us an array (it reads and writes 4 bytes a
 // slot, the reads of a tile within its own lines).  Up to kFewSlots slots, all
 // arrays are gathered by one launch and brought back by one copy, since there
 // every launch and copy counts more than the bytes; beyond, one array at a
