@@ -102,7 +102,8 @@ static std::map<unsigned, Bar> bar_of;
 static std::vector<Copy> held;   // started, not landed
 static int hold_from = 1 << 30;  // copies from this one on are held
 static int started = 0, started_late = 0, asked = 0;
-static std::atomic<bool> given_up{false};  // by the lane that starts the copies, the first to lose patience here
+static std::atomic<bool> given_up{false};  // a wait of the lane that starts the copies has run out
+static thread_local int polls = 0;         // of the running wait
 static bool land_late = false;
 static thread_local unsigned long long now = 1;
 static void land(const Copy& c) {
@@ -119,10 +120,8 @@ static unsigned fdog_smem_addr(const void* p) {
 static void fdog_bar_init(unsigned bars, int n) {
     for (int s = 0; s < n; ++s) bar_of[bars + 8u * s] = Bar();
 }
-static InstCtl ctl;
 static void fdog_bar_expect(unsigned bar, unsigned bytes) {
     std::lock_guard<std::mutex> lk(mu);
-    if (ctl.error) given_up = true;
     bar_of[bar].pending += bytes;
 }
 static void fdog_bulk_copy(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
@@ -132,16 +131,27 @@ static void fdog_bulk_copy(unsigned dst, const void* src, unsigned bytes, unsign
     if (started++ >= hold_from) held.push_back(c);
     else land(c);
 }
+static InstCtl ctl;
 static bool fdog_bar_done(unsigned bar, unsigned parity) {
     std::lock_guard<std::mutex> lk(mu);
-    if (threadIdx.x == 0 && ctl.error) given_up = true;
     if (given_up && land_late && threadIdx.x == 0 && ++asked == 3) {
         for (const Copy& c : held) land(c);
         held.clear();
     }
-    return bar_of[bar].phase != parity;
+    const bool done = bar_of[bar].phase != parity;
+    if (done) polls = 0;
+    return done;
 }
-static unsigned long long fdog_now() { return now += threadIdx.x == 0 || given_up ? 300000000ull : 100000ull; }
+// 0.3 s a poll for the lane that starts the copies, whose waits so end with their fifth; the others' time stands still
+// until one of them has
+static unsigned long long fdog_now() {
+    if (threadIdx.x != 0) return now += given_up ? 300000000ull : 0ull;
+    if (++polls == 5) {
+        polls = 0;
+        given_up = true;
+    }
+    return now += 300000000ull;
+}
 static std::atomic<int> wrong{0};
 static int k_of[2] = {3, 2};
 #define FDOG_BULK_DISPATCH(MODE) \
